@@ -73,9 +73,9 @@ def listed():
         # small batches at interactive rates: one replayed graph
         {"name": "batches_replay", "kind": "replay", "variant": "page_array", "staging": False, "n_batches": 32,
          "log_lo": 8, "log_hi": 13, "hi": 4096, "heap_mib": 1024},
-        # a serving loop whose memory pressure binds the admission
-        {"name": "serving_loop", "kind": "serve", "variant": "page_array", "steps": 400, "rate": 2000,
-         "median_kib": 4096, "slots": 4096, "heap_mib": 16384},
+        # a serving loop at a load that now and then fills its slots, from the first arrival to the last free
+        {"name": "serving_loop", "kind": "serve", "variant": "page_array", "steps": 400, "rate": 5500,
+         "median_kib": 1024, "slots": 4096, "heap_mib": 16384},
         # a scale-free graph arriving edge by edge
         {"name": "graph_growth", "kind": "graph", "variant": "page_array", "vertices": 1 << 18, "edges": 1 << 22,
          "heap_mib": 2048},
@@ -112,9 +112,11 @@ def draw(rng):
         return {"kind": kind, "variant": variant, "staging": staging, "n_batches": _log(rng, 8, 64), "log_lo": 6,
                 "log_hi": rng.randint(10, 13), "hi": _log(rng, 64, 8192), "heap_mib": 1024}
     if kind == "serve":
-        return {"kind": kind, "variant": rng.choice(("page_array", "page_array", "page_varray", "chunk_array")),
-                "steps": _log(rng, 50, 300), "rate": rng.randint(200, 2000), "median_kib": _log(rng, 128, 4096),
-                "slots": _log(rng, 256, 4096), "heap_mib": 8192}
+        case = {"kind": kind, "variant": rng.choice(("page_array", "page_array", "page_varray", "chunk_array")),
+                "steps": _log(rng, 50, 400), "median_kib": _log(rng, 64, 1024), "slots": _log(rng, 256, 4096),
+                "heap_mib": 16384}
+        case["rate"] = round(100 * case["slots"] / _mean_blocks(case) * rng.uniform(0.2, 0.95))   # of what the slots take
+        return case
     return {"kind": "graph", "variant": rng.choice(("page_array", "page_array", "page_varray", "chunk_array")),
             "vertices": _log(rng, 1 << 14, 1 << 18), "edges": _log(rng, 1 << 16, 1 << 21), "heap_mib": 2048}
 
@@ -137,12 +139,29 @@ def _batches(case, seed):
 
 
 def _sessions(case, seed):
-    """workloads.serving_workload for a given number of sessions, so that the results of every seed have one shape."""
+    """Sessions of workloads.serving_workload's kind that a run of `steps` steps serves to their end: a given number
+    of them, arriving in the first 40 % of the steps and growing for at most 40 % of them."""
     r = W.rng(seed)
-    n = int(case["rate"] * 0.01 * case["steps"])
-    arrive = np.sort(r.integers(0, case["steps"], n)).astype(np.uint32)
+    span = case["steps"] * 2 // 5
+    n = int(case["rate"] * 0.01 * span)
+    arrive = np.sort(r.integers(0, span, n)).astype(np.uint32)
     size = r.lognormal(math.log(case["median_kib"] << 10), 1.0, n)
-    return arrive, np.clip(np.ceil(size / BLOCK), 1, 2048).astype(np.uint32)
+    return arrive, np.clip(np.ceil(size / BLOCK), 1, span).astype(np.uint32)
+
+
+def _mean_blocks(case):
+    """Mean of ceil(lognormal / BLOCK) clipped to the 40 % of the steps, by quadrature over the quantiles."""
+    q = [(i + 0.5) / 400 for i in range(400)]
+    z = [math.sqrt(2.0) * _erfinv(2 * p - 1) for p in q]
+    span = case["steps"] * 2 // 5
+    return sum(min(max(math.ceil((case["median_kib"] << 10) * math.exp(t) / BLOCK), 1), span) for t in z) / len(z)
+
+
+def _erfinv(x):
+    """Winitzki's approximation (2 parts in 1000), enough for an expected size."""
+    a, ln = 0.147, math.log(1 - x * x)
+    t = 2 / (math.pi * a) + ln / 2
+    return math.copysign(math.sqrt(math.sqrt(t * t - ln / a) - t), x)
 
 
 def _edges(case, seed):
@@ -168,8 +187,8 @@ def prepare(case, seed):
     elif kind == "serve":
         arrive, blocks = _sessions(case, seed)
         st["cap"] = int(0.95 * (case["heap_mib"] * MIB // BLOCK))
-        st["run"] = serving.ServeRun(arrive, blocks, n_slots=case["slots"], max_blocks=2048, steps=case["steps"],
-                                     seed=st["seed"], block_bytes=BLOCK)
+        st["run"] = serving.ServeRun(arrive, blocks, n_slots=case["slots"], max_blocks=int(blocks.max(initial=1)),
+                                     steps=case["steps"], seed=st["seed"], block_bytes=BLOCK)
     else:
         src, dst = _edges(case, seed)
         st["run"] = graph.GraphRun(src, dst, case["vertices"])
@@ -239,12 +258,8 @@ def work(case):
         mean = (2.0 ** hi - 2.0 ** lo) / ((hi - lo) * math.log(2))
         return {"bytes": case["n_batches"] * (40 + mean * (4 + (4 + case["hi"]) / 2)), "flops": 0}
     if kind == "serve":
-        # one block per active session and step: the sessions of the steps before, until the heap or the slots bind
-        blocks = min(2048.0, case["median_kib"] * 1024 * math.exp(0.5) / BLOCK)
-        cap = min(case["slots"], 0.95 * case["heap_mib"] * MIB / BLOCK / blocks)
-        per_step = case["rate"] * 0.01
-        active = sum(min(cap, per_step * min(t + 1, blocks)) for t in range(case["steps"]))
-        return {"bytes": active * (BLOCK + 8), "flops": 0}
+        n = int(case["rate"] * 0.01 * (case["steps"] * 2 // 5))
+        return {"bytes": n * (48 + _mean_blocks(case) * (BLOCK + 8)), "flops": 0}
     # the edges read, the rows written, read and written again in order, the vertex records
     return {"bytes": case["edges"] * (8 + 4 + 8 + 8) + case["vertices"] * 40, "flops": 0}
 
