@@ -92,6 +92,7 @@ static ouro_status init_state(ouro_heap *H, cudaStream_t s) {
   ouro_heap_dev &d = H->d;
   OURO_CUDA(cudaMemsetAsync(H->meta + H->off_glob, 0, sizeof(ouro_glob), s));
   OURO_CUDA(cudaMemsetAsync(H->meta + H->off_stats, 0, H->stats_words * 8, s));
+  OURO_CUDA(cudaMemsetAsync(H->meta + H->off_work, 0, OURO_WORK_SLOTS * 128, s));
   k_init_qhdr<<<OURO_MAX_CLASSES, 128, 0, s>>>(d);   /* every class, runs above one chunk too */
   OURO_LAUNCHED();
   const int grid = 4 * sm_count();

@@ -14,8 +14,8 @@
 /* virtualized-array directories also span positions that are waiting for a
  * producer or in flight (more than twice the resident threads of 152 SMs) */
 #define OURO_VA_SLACK (1ull << 20)
-/* work counters of fused rounds: one per launch in flight on a heap, each on
- * its own 128-byte line, handed out round robin */
+/* work slots of fused rounds: one per launch in flight on a heap, each on its
+ * own 128-byte line, handed out round robin; zero between launches */
 #define OURO_WORK_SLOTS 64
 
 struct ouro_heap {
@@ -38,6 +38,20 @@ extern thread_local int g_last_cuda_error;
 ouro_status cuda_fail(cudaError_t e);
 void count_launch(unsigned n = 1);
 int sm_count();
+
+/* Requests that a warp of the fused kernels takes at a time, 2^0 .. 2^5, for
+ * n requests on `warps` resident warps.  A warp walks its larger blocks one
+ * after another and every allocator step is a chain of L2 round trips, so up
+ * to eight requests per warp go out as one task each (32 batches of 256 to
+ * 8192 requests: 62 us a round with tasks of 32, 11 so).  Beyond that a warp
+ * gets at least four tasks, so that the last ones fill the gaps, of at least
+ * eight requests, which share their queue atomics. */
+inline unsigned round_task(unsigned long long n, unsigned long long warps) {
+  unsigned t = 1;
+  while (t < 8 && t * warps < n) t *= 2;
+  while (t < 32 && 8 * t * warps <= n) t *= 2;
+  return t;
+}
 }  // namespace host
 }  // namespace ouro
 

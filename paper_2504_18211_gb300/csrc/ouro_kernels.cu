@@ -354,28 +354,84 @@ __global__ void __launch_bounds__(256) k_batch_malloc_cblk(ouro_heap_dev h, cons
   }
 }
 
+/* mode 0 of k_pattern: one word per block, a lane each; a thread's four
+ * pointers, then its four words, in flight together.  Every word is a sector
+ * of its own, so what bounds it is scattered sectors, not bytes. */
 template <int OP>
-__global__ void k_pattern(void *const *ptrs, const uint32_t *sizes, size_t n, uint32_t seed, int mode,
-                          ouro_check *out) {
+__device__ __forceinline__ void pattern_ids(void *const *ptrs, size_t n, payload_acc &a, unsigned long long &nulls) {
+  const size_t threads = (size_t)gridDim.x * blockDim.x;
+  for (size_t i0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i0 < n; i0 += 4 * threads) {
+    uint32_t *p[4];
+    uint32_t v[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) p[k] = i0 + k * threads < n ? static_cast<uint32_t *>(ptrs[i0 + k * threads]) : nullptr;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      if (OP & PAY_WRITE) {
+        if (p[k]) *p[k] = (uint32_t)(i0 + k * threads);
+      } else {
+        v[k] = p[k] ? __ldcg(p[k]) : 0u;
+      }
+    }
+    if (OP & PAY_CHECK) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        if (p[k]) {
+          a.mism += v[k] != (uint32_t)(i0 + k * threads);
+          a.fold(v[k]);
+          a.words++;
+        } else if (i0 + k * threads < n) {
+          nulls++;
+        }
+      }
+    }
+  }
+}
+
+/* The requests are cut into tasks: the first `heads` of them of 32 requests,
+ * the rest of `task` requests (a power of two of at most 32).  The tasks are
+ * dealt to the blocks in turn, and a block's warps pull the block's tasks from
+ * a shared-memory counter: long tasks first, which share a row of small blocks
+ * among 32 requests, short ones last, so that the warps end together.  With
+ * fixed 32-request strides a warp had 3 or 4 of them at 2^20 requests and the
+ * kernel waited for the fours. */
+template <int OP>
+__global__ void __launch_bounds__(256) k_pattern(void *const *ptrs, const uint32_t *sizes, size_t n, uint32_t seed,
+                                                 int mode, size_t heads, unsigned task, ouro_check *out) {
+  __shared__ unsigned s_next;
+  if (threadIdx.x == 0) s_next = 0;
+  __syncthreads();
   payload_acc a;
   unsigned long long nulls = 0;
-  const size_t warps = ((size_t)gridDim.x * blockDim.x) >> 5;
-  const size_t wid = (((size_t)blockIdx.x * blockDim.x) + threadIdx.x) >> 5;
-  for (size_t base = wid * 32; base < n; base += warps * 32) {
-    const size_t i = base + (threadIdx.x & 31);
-    unsigned char *p = i < n ? static_cast<unsigned char *>(ptrs[i]) : nullptr;
-    const uint32_t sz = i < n ? sizes[i] : 0;
-    if (i < n && !p) nulls++;
-    warp_payload<OP>(p, sz, (uint32_t)i, seed, mode, a);
+  if (mode == 0) {
+    pattern_ids<OP>(ptrs, n, a, nulls);
+  } else {
+    const unsigned lane = threadIdx.x & 31;
+    const size_t tasks = heads + (n - 32 * heads + task - 1) / task;
+    for (;;) {
+      unsigned t = 0;
+      if (lane == 0) t = atomicAdd(&s_next, 1u);
+      t = __shfl_sync(0xffffffffu, t, 0);
+      const size_t k = (size_t)t * gridDim.x + blockIdx.x;
+      if (k >= tasks) break;
+      const size_t i = (k < heads ? 32 * k : 32 * heads + (k - heads) * task) + lane;
+      const bool mine = lane < (k < heads ? 32u : task) && i < n;
+      unsigned char *p = mine ? static_cast<unsigned char *>(ptrs[i]) : nullptr;
+      const uint32_t sz = mine ? sizes[i] : 0;
+      if (mine && !p) nulls++;
+      warp_payload<OP>(p, sz, (uint32_t)i, seed, 1, a);
+    }
   }
   if (OP & PAY_CHECK) flush_acc(a, nulls, out);
 }
 
-/* one whole round per thread: malloc, write, read back, free.  Warps pull
- * 32 requests at a time from the launch's work counter, so blocks of
+/* one whole round per thread: malloc, write, read back, free.  Warps take
+ * `task` requests (a power of two of at most 32) at a time: warp w of the
+ * grid the w-th task, then tasks from the launch's work slot, so blocks of
  * uneven sizes balance across warps and the round ends within one task of
- * the last byte.  STAGE: the warp's freed pages serve its next mallocs of
- * the same class from shared memory (page queues, heap option `staging`). */
+ * the last byte.  The lanes past `task` ask for nothing but help their
+ * warp's carves and payload.  STAGE: the warp's freed pages serve its next
+ * mallocs of the same class from shared memory (heap option `staging`). */
 #ifndef OURO_FUSED_MIN_BLOCKS
 #define OURO_FUSED_MIN_BLOCKS 4   /* resident blocks of 256 per SM the fused round is compiled for */
 #endif
@@ -383,27 +439,23 @@ __global__ void k_pattern(void *const *ptrs, const uint32_t *sizes, size_t n, ui
  * (128 registers a thread) instead of spilling at 64 */
 template <int V, bool STAGE>
 __global__ void __launch_bounds__(256, ouro_page_queues(V) ? OURO_FUSED_MIN_BLOCKS : 2) k_round_fused(ouro_heap_dev h, const uint32_t *sizes, size_t n,
-                                                     uint32_t seed, int mode, ouro_check *out, void **ptrs,
-                                                     unsigned long long *work) {
+                                                     uint32_t seed, int mode, unsigned task, ouro_check *out,
+                                                     void **ptrs, work_slot *work) {
   __shared__ ouro_block_ctx<8> ctx;
   if (STAGE) ouro_block_begin(ctx);
   payload_acc a;
   unsigned long long nulls = 0;
   const unsigned lane = threadIdx.x & 31;
-  for (;;) {
-    unsigned long long base = 0;
-    if (lane == 0) base = atomicAdd(work, 32ull);
-    base = __shfl_sync(0xffffffffu, base, 0);
-    if (base >= n) break;
+  const unsigned long long first = (unsigned long long)gridDim.x * (blockDim.x >> 5) * task;   /* tasks not handed out */
+  unsigned long long base = (unsigned long long)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * task;
+  while (base < n) {
     const size_t i = base + lane;
-    const uint32_t sz = i < n ? sizes[i] : 0;
-    unsigned char *p = nullptr;
-    if (STAGE) {
-      p = static_cast<unsigned char *>(stage_malloc_v<V>(ctx, h, sz, i < n));
-    } else if (i < n) {
-      p = static_cast<unsigned char *>(malloc_v<V>(h, sz));
-    }
-    if (i < n) {
+    const bool mine = lane < task && i < n;
+    const uint32_t sz = mine ? sizes[i] : 0;
+    unsigned char *p;
+    if (STAGE) p = static_cast<unsigned char *>(stage_malloc_v<V>(ctx, h, sz, mine));
+    else p = static_cast<unsigned char *>(malloc_v<V>(h, sz, mine));
+    if (mine) {
       if (!p) nulls++;
       if (ptrs) ptrs[i] = p;
     }
@@ -413,11 +465,14 @@ __global__ void __launch_bounds__(256, ouro_page_queues(V) ? OURO_FUSED_MIN_BLOC
     /* staged: the class of each block is known here, so the free skips the
      * chunk-table lookup (one L2 round trip per task off the warp's chain) */
     if (STAGE) ouro::detail::stage_free<V, 8>(ctx, h, p, __activemask(), p ? size_class(h, sz) : -1);
-    else if (i < n) free_v<V>(h, p);
+    else free_v<V>(h, p);
     __syncwarp();
+    if (first >= n) break;
+    if (lane == 0) base = first + atomicAdd(&work->next, (unsigned long long)task);
+    base = __shfl_sync(0xffffffffu, base, 0);
   }
   if (STAGE) ouro_block_end_v<V>(ctx, h);
-  flush_acc(a, nulls, out);
+  finish_acc(a, nulls, work, out);
 }
 
 #if OURO_SHARD_ENTRIES
@@ -432,11 +487,45 @@ int occupancy_grid(K kernel, int block) {
   return per_sm * ouro::host::sm_count();
 }
 
+/* the largest power of two up to 32 that leaves every one of `warps` warps
+ * `per` tasks of n requests (1 at least) */
+inline unsigned task_size(size_t n, size_t warps, int per) {
+  unsigned t = 1;
+  while (t < 32 && 2 * t * warps * per <= n) t *= 2;
+  return t;
+}
+
 inline int grid_for(size_t n, int block, int cap) {
   size_t g = (n + block - 1) / block;
   if (g < 1) g = 1;
   return (int)(g < (size_t)cap ? g : (size_t)cap);
 }
+
+#if OURO_SHARD_ENTRIES
+/* How k_pattern cuts n requests: whole rounds of 32-request tasks for all
+ * resident warps while they cover at most 7/8 of the requests, then tasks
+ * that give every warp about four; a batch with less than a round, tasks of
+ * an eighth of a warp's share (1024 blocks of 1000 B: one each).  Measured on
+ * malloc + write + check + free of 2^20 size-sweep requests: fixed strides of
+ * 32 697 us; all tasks of 32 / 16 / 8 / 4 requests 636 / 622 / 609 / 607; so
+ * 607.  3 * 2^18 blocks of 64 B with all tasks of 8: 21 us each way, bound by
+ * the instructions per task; so 17 and 20. */
+struct pattern_shape {
+  size_t heads = 0;
+  unsigned task = 32;
+  int grid;
+  pattern_shape(size_t n, int mode, int block, int cap) {
+    const size_t warps = (size_t)cap * (block / 32);
+    size_t tasks = (n + 31) / 32;
+    if (mode) {
+      heads = n / 8 * 7 / (32 * warps) * warps;
+      task = task_size(n - 32 * heads, warps, heads ? 4 : 8);
+      tasks = heads + (n - 32 * heads + task - 1) / task;
+    }
+    grid = grid_for(tasks * 32, block, cap);
+  }
+};
+#endif
 
 }  // namespace
 
@@ -530,18 +619,22 @@ ouro_status batch_free(ouro_heap *H, void *const *d_ptrs, size_t n, cudaStream_t
   return OURO_OK;
 }
 
-template <int V>
-ouro_status round_fused(ouro_heap *H, const uint32_t *d_sizes, size_t n, uint32_t seed, int mode, ouro_check *d_out,
-                        void **d_ptrs, unsigned long long *work, cudaStream_t s) {
-  const int block = 256;
-  if (H->d.staging)
-    k_round_fused<V, true><<<grid_for(n, block, occupancy_grid(k_round_fused<V, true>, block)), block, 0, s>>>(
-        H->d, d_sizes, n, seed, mode, d_out, d_ptrs, work);
-  else
-    k_round_fused<V, false><<<grid_for(n, block, occupancy_grid(k_round_fused<V, false>, block)), block, 0, s>>>(
-        H->d, d_sizes, n, seed, mode, d_out, d_ptrs, work);
+template <int V, bool STAGE>
+ouro_status round_fused_form(ouro_heap *H, const uint32_t *d_sizes, size_t n, uint32_t seed, int mode,
+                             ouro_check *d_out, void **d_ptrs, void *work, cudaStream_t s) {
+  const int block = 256, cap = occupancy_grid(k_round_fused<V, STAGE>, block);
+  const unsigned task = ouro::host::round_task(n, (size_t)cap * (block / 32));
+  k_round_fused<V, STAGE><<<grid_for((n + task - 1) / task * 32, block, cap), block, 0, s>>>(
+      H->d, d_sizes, n, seed, mode, task, d_out, d_ptrs, static_cast<work_slot *>(work));
   OURO_LAUNCHED();
   return OURO_OK;
+}
+
+template <int V>
+ouro_status round_fused(ouro_heap *H, const uint32_t *d_sizes, size_t n, uint32_t seed, int mode, ouro_check *d_out,
+                        void **d_ptrs, void *work, cudaStream_t s) {
+  return H->d.staging ? round_fused_form<V, true>(H, d_sizes, n, seed, mode, d_out, d_ptrs, work, s)
+                      : round_fused_form<V, false>(H, d_sizes, n, seed, mode, d_out, d_ptrs, work, s);
 }
 
 #define INST_BATCH_MALLOC(PRE, V) \
@@ -550,7 +643,7 @@ ouro_status round_fused(ouro_heap *H, const uint32_t *d_sizes, size_t n, uint32_
   PRE template ouro_status batch_free<V>(ouro_heap *, void *const *, size_t, cudaStream_t);
 #define INST_ROUND_FUSED(PRE, V)                                                                                 \
   PRE template ouro_status round_fused<V>(ouro_heap *, const uint32_t *, size_t, uint32_t, int, ouro_check *, \
-                                          void **, unsigned long long *, cudaStream_t);
+                                          void **, void *, cudaStream_t);
 OURO_SHARD_INSTANTIATE(INST_BATCH_MALLOC)
 OURO_SHARD_INSTANTIATE(INST_BATCH_FREE)
 OURO_SHARD_INSTANTIATE(INST_ROUND_FUSED)
@@ -579,8 +672,8 @@ extern "C" ouro_status ouro_pattern_write(void *const *d_ptrs, const uint32_t *d
   if (mode != 0 && mode != 1) return OURO_EINVAL;
   if (!n) return OURO_OK;
   const int block = 256;
-  const int g = grid_for((n + 31) / 32 * 32, block, occupancy_grid(k_pattern<PAY_WRITE>, block));
-  k_pattern<PAY_WRITE><<<g, block, 0, S(stream)>>>(d_ptrs, d_sizes, n, seed, mode, nullptr);
+  const pattern_shape sh(n, mode, block, occupancy_grid(k_pattern<PAY_WRITE>, block));
+  k_pattern<PAY_WRITE><<<sh.grid, block, 0, S(stream)>>>(d_ptrs, d_sizes, n, seed, mode, sh.heads, sh.task, nullptr);
   OURO_LAUNCHED();
   return OURO_OK;
 }
@@ -592,8 +685,8 @@ extern "C" ouro_status ouro_pattern_check(void *const *d_ptrs, const uint32_t *d
   OURO_CUDA(cudaMemsetAsync(d_out, 0, sizeof(ouro_check), S(stream)));
   if (!n) return OURO_OK;
   const int block = 256;
-  const int g = grid_for((n + 31) / 32 * 32, block, occupancy_grid(k_pattern<PAY_CHECK>, block));
-  k_pattern<PAY_CHECK><<<g, block, 0, S(stream)>>>(d_ptrs, d_sizes, n, seed, mode, d_out);
+  const pattern_shape sh(n, mode, block, occupancy_grid(k_pattern<PAY_CHECK>, block));
+  k_pattern<PAY_CHECK><<<sh.grid, block, 0, S(stream)>>>(d_ptrs, d_sizes, n, seed, mode, sh.heads, sh.task, d_out);
   OURO_LAUNCHED();
   return OURO_OK;
 }
@@ -602,13 +695,14 @@ extern "C" ouro_status ouro_round_fused(ouro_heap *H, const uint32_t *d_sizes, s
                                         ouro_check *d_out, void **d_ptrs, void *stream) {
   if (!H || !d_out || (n && !d_sizes)) return OURO_EINVAL;
   if (mode != 0 && mode != 1) return OURO_EINVAL;
-  OURO_CUDA(cudaMemsetAsync(d_out, 0, sizeof(ouro_check), S(stream)));
-  if (!n) return OURO_OK;
-  /* this launch's work counter: a slot of the heap's ring, zeroed on the
-   * launch's stream (launches in flight at once on one heap: up to 64) */
+  if (!n) {
+    OURO_CUDA(cudaMemsetAsync(d_out, 0, sizeof(ouro_check), S(stream)));
+    return OURO_OK;
+  }
+  /* this launch's work slot, one of the heap's ring (launches in flight at
+   * once on one heap: up to 64); the launch leaves it zero */
   const unsigned slot = __atomic_fetch_add(&H->work_seq, 1u, __ATOMIC_RELAXED) % OURO_WORK_SLOTS;
-  unsigned long long *work = (unsigned long long *)(H->meta + H->off_work + (size_t)slot * 128);
-  OURO_CUDA(cudaMemsetAsync(work, 0, 8, S(stream)));
+  void *work = H->meta + H->off_work + (size_t)slot * 128;
   OURO_DISPATCH(H->d.variant,
                 return ouro::launch::round_fused<V>(H, d_sizes, n, seed, mode, d_out, d_ptrs, work, S(stream)));
 }

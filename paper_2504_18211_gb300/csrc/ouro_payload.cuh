@@ -100,22 +100,37 @@ struct payload_acc {
   }
 };
 
-/* Warp-cooperative payload over the 32 blocks of a warp, one block at a
- * time: all 32 lanes stride over the block's 16-byte units, several units in
- * flight per lane.  Every lane of the warp must call (a lane without a block
- * passes p = null).
+/* Warp-cooperative payload over the blocks held by the lanes of a warp (every
+ * lane calls; a lane without a block passes p = null).
  *   WRITE:  store the pattern.
  *   CHECK:  read back, compare, fold the checksums into a.
- *   FUSED:  write the block, then (after __syncwarp) read it back through L2
- *           with every lane checking the units its neighbour wrote.
+ *   FUSED:  write, then (after __syncwarp) read back through L2 with every
+ *           lane checking what a neighbour wrote.
  * mode 0: word 0 = tid.  mode 1: floor(size/4) words key + w*GOLD, then the
- * low size%4 bytes of word floor(size/4). */
+ * low size%4 bytes of word floor(size/4).
+ *
+ * A block is cut into 16-byte units and a rest of up to 15 bytes.  What
+ * bounds the payload of small blocks is the chain of L2 round trips, so the
+ * blocks of up to pay_flat units are laid end to end and the 32 lanes stride
+ * over the whole row of units, four loads in flight per lane: a row of 32
+ * blocks of 16 B is one store and one load per lane instead of 32 round
+ * trips with 31 lanes idle (3 * 2^18 blocks of 64 B: write 45 -> 17 us, check
+ * 88 -> 20 us; a fused round of 10,240 blocks of 16 B 37 -> 12 us).  Larger
+ * blocks fill the warp by themselves and go one at a time, so that a block is
+ * read back while L2 still holds it (laying all 32 end to end pushed most of
+ * the read-back out to DRAM).  The rests are done by the lanes that hold the
+ * blocks, all at once, instead of by one lane block after block. */
 enum { PAY_WRITE = 1, PAY_CHECK = 2, PAY_FUSED = 3 };
+/* units of the largest block that goes into the row: where the row writes and
+ * reads back, its longer stretch between the two costs a little on a full
+ * chip (2^20 sweep: 16 units 315 us, 32 units 317, 64 units 326), so it stays
+ * shorter than where a kernel does one of the two */
+__host__ __device__ constexpr unsigned pay_flat(int op) { return op == PAY_FUSED ? 16u : 64u; }
 
-__device__ __forceinline__ uint4 pat4(uint32_t key, uint32_t w0) {
-  return make_uint4(key + w0 * OURO_GOLD, key + (w0 + 1) * OURO_GOLD, key + (w0 + 2) * OURO_GOLD,
-                    key + (w0 + 3) * OURO_GOLD);
+__device__ __forceinline__ uint4 pat4(uint32_t v) {
+  return make_uint4(v, v + OURO_GOLD, v + 2u * OURO_GOLD, v + 3u * OURO_GOLD);
 }
+__device__ __forceinline__ uint4 pat4(uint32_t key, uint32_t w0) { return pat4(key + w0 * OURO_GOLD); }
 
 __device__ __forceinline__ void check4(const uint4 &got, const uint4 &want, payload_acc &a) {
   a.mism += (got.x != want.x) + (got.y != want.y) + (got.z != want.z) + (got.w != want.w);
@@ -123,38 +138,135 @@ __device__ __forceinline__ void check4(const uint4 &got, const uint4 &want, payl
   a.s += (unsigned long long)got.x + got.y + got.z + got.w;
 }
 
-/* words [4*units, nw) and the tail bytes of one block: one lane */
+/* Payload units pass through L2 once, so stores and loads carry the
+ * evict_first policy: a unit that was read back is the next to leave L2, and
+ * the dirty lines go out to HBM about in the order they were written, instead
+ * of in the order of an LRU over all of L2 (which also held the allocator's
+ * slots and tables).  2^20 fused size-sweep round: 326 -> 315 us; the policy
+ * on the stores alone 351 us (the read-back renewed the lines), on the loads
+ * alone 330.  ld.global.cg reads L2, past any line of L1. */
+__device__ __forceinline__ unsigned long long stream_policy() {
+  unsigned long long pol;
+  asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
+  return pol;
+}
+__device__ __forceinline__ void st_stream(uint4 *p, const uint4 &v, unsigned long long pol) {
+  asm volatile("st.global.L2::cache_hint.v4.u32 [%0], {%1, %2, %3, %4}, %5;" ::"l"(p), "r"(v.x), "r"(v.y), "r"(v.z),
+               "r"(v.w), "l"(pol)
+               : "memory");
+}
+__device__ __forceinline__ uint4 ld_stream(const uint4 *p, unsigned long long pol) {
+  uint4 v;
+  asm volatile("ld.global.cg.L2::cache_hint.v4.u32 {%0, %1, %2, %3}, [%4], %5;"
+               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p), "l"(pol) : "memory");
+  return v;
+}
+
+/* the words past the last whole unit and the tail bytes of one block, by one
+ * lane; the loads of the read-back are independent of each other */
 template <bool WRITE>
-__device__ void block_rest(unsigned char *bp, uint32_t key, uint32_t nw, uint32_t tail, payload_acc &a) {
-  uint32_t *wp = reinterpret_cast<uint32_t *>(bp);
-  for (uint32_t w = nw & ~3u; w < nw; ++w) {
-    const uint32_t want = key + w * OURO_GOLD;
-    if (WRITE) wp[w] = want;
-    else {
-      uint32_t got = __ldcg(wp + w);
-      a.mism += got != want;
-      a.fold(got);
+__device__ __forceinline__ void block_rest(unsigned char *bp, uint32_t key, uint32_t size, payload_acc &a) {
+  const uint32_t nw = size >> 2, tail = size & 3, w0 = nw & ~3u, k = nw & 3u;
+  uint32_t *wp = reinterpret_cast<uint32_t *>(bp) + w0;
+  unsigned char *tb = bp + 4ull * nw;
+  const uint32_t v = key + nw * OURO_GOLD;
+  if (WRITE) {
+#pragma unroll
+    for (uint32_t w = 0; w < 3; ++w)
+      if (w < k) wp[w] = key + (w0 + w) * OURO_GOLD;
+#pragma unroll
+    for (uint32_t b = 0; b < 3; ++b)
+      if (b < tail) tb[b] = (unsigned char)(v >> (8 * b));
+  } else {
+    uint32_t g[3], t[3];
+#pragma unroll
+    for (uint32_t w = 0; w < 3; ++w) g[w] = w < k ? __ldcg(wp + w) : 0u;
+#pragma unroll
+    for (uint32_t b = 0; b < 3; ++b) t[b] = b < tail ? __ldcg(tb + b) : 0u;
+#pragma unroll
+    for (uint32_t w = 0; w < 3; ++w) {
+      a.mism += w < k && g[w] != key + (w0 + w) * OURO_GOLD;
+      a.fold(g[w]);
     }
-  }
-  if (tail) {
-    const uint32_t v = key + nw * OURO_GOLD;
-    unsigned char *tb = bp + 4ull * nw;
-    if (WRITE) {
-      for (uint32_t b = 0; b < tail; ++b) tb[b] = (unsigned char)(v >> (8 * b));
-    } else {
-      uint32_t got = 0;
-      for (uint32_t b = 0; b < tail; ++b) {
-        unsigned char gb = __ldcg(tb + b);
-        a.mism += gb != (unsigned char)(v >> (8 * b));
-        got |= (uint32_t)gb << (8 * b);
-      }
-      a.fold(got);
-    }
+#pragma unroll
+    for (uint32_t b = 0; b < 3; ++b) a.mism += b < tail && t[b] != ((v >> (8 * b)) & 0xFFu);
+    a.fold(t[0] | t[1] << 8 | t[2] << 16);
   }
 }
 
+/* Lane whose block holds unit f of the row: the number of lanes whose
+ * running count incl does not pass f (31 at most). */
+__device__ __forceinline__ unsigned row_owner(unsigned incl, unsigned f) {
+  unsigned j = 0;
+#pragma unroll
+  for (unsigned s = 16; s; s >>= 1)
+    if (__shfl_sync(0xffffffffu, incl, j + s - 1) <= f) j += s;
+  return j;
+}
+
+/* The row of small blocks (n_units > 0 for a lane whose block is in it) and
+ * every block's rest.  Out of line: its registers (four loads in flight and
+ * their places in the row) stay out of the allocating kernels' budget. */
 template <int OP>
-__device__ void warp_payload(unsigned char *p, uint32_t size, uint32_t tid, uint32_t seed, int mode, payload_acc &a) {
+__device__ __noinline__ payload_acc payload_row(unsigned char *p, uint32_t size, uint32_t key, uint32_t n_units) {
+  constexpr unsigned FULL = 0xffffffffu;
+  const unsigned lane = laneid();
+  const unsigned rd = OP == PAY_FUSED ? (lane + 1) & 31 : lane;   /* lane whose units this lane checks */
+  const unsigned long long pol = stream_policy();
+  payload_acc a;
+  uint32_t incl = n_units;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(FULL, incl, o);
+    if ((int)lane >= o) incl += y;
+  }
+  const uint32_t total = __shfl_sync(FULL, incl, 31);
+  const uint32_t excl = incl - n_units;
+  /* unit f of the row, in this lane's block: address row_p + 16 f, first word row_k + 4 f * GOLD */
+  const unsigned long long row_p = reinterpret_cast<unsigned long long>(p) - 16ull * excl;
+  const uint32_t row_k = key - 4u * excl * OURO_GOLD;
+  if (OP & PAY_WRITE) {
+    for (uint32_t f0 = 0; f0 < total; f0 += 32) {
+      const uint32_t f = f0 + lane;
+      const unsigned j = row_owner(incl, f);
+      const unsigned long long bp = __shfl_sync(FULL, row_p, j);
+      const uint32_t v = __shfl_sync(FULL, row_k, j);
+      if (f < total) st_stream(reinterpret_cast<uint4 *>(bp + 16ull * f), pat4(v, 4 * f), pol);
+    }
+    if (size & 15) block_rest<true>(p, key, size, a);
+  }
+  if (OP == PAY_FUSED) __syncwarp();
+  if (OP & PAY_CHECK) {
+    for (uint32_t f0 = 0; f0 < total; f0 += 128) {
+      uint4 g[4];
+      uint32_t v[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const uint32_t f = f0 + 32 * k + rd;
+        const unsigned j = row_owner(incl, f);
+        const unsigned long long bp = __shfl_sync(FULL, row_p, j);
+        v[k] = __shfl_sync(FULL, row_k, j) + 4 * f * OURO_GOLD;
+        if (f < total) g[k] = ld_stream(reinterpret_cast<const uint4 *>(bp + 16ull * f), pol);
+      }
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (f0 + 32 * k + rd < total) check4(g[k], pat4(v[k]), a);
+    }
+    if (OP == PAY_FUSED) {
+      const unsigned long long np = __shfl_sync(FULL, reinterpret_cast<unsigned long long>(p), rd);
+      const uint32_t ns = __shfl_sync(FULL, size, rd), nk = __shfl_sync(FULL, key, rd);
+      if (ns & 15) block_rest<false>(reinterpret_cast<unsigned char *>(np), nk, ns, a);
+    } else if (size & 15) {
+      block_rest<false>(p, key, size, a);
+    }
+  }
+  return a;
+}
+
+template <int OP>
+__device__ __forceinline__ void warp_payload(unsigned char *p, uint32_t size, uint32_t tid, uint32_t seed, int mode,
+                                             payload_acc &a) {
+  constexpr unsigned FULL = 0xffffffffu;
   const unsigned lane = laneid();
   if (mode == 0) {
     if (p) {
@@ -170,44 +282,53 @@ __device__ void warp_payload(unsigned char *p, uint32_t size, uint32_t tid, uint
     return;
   }
   const uint32_t key = fmix32(seed ^ (tid * OURO_GOLD));
-  const unsigned rd = OP == PAY_FUSED ? (lane + 1) & 31 : lane;   /* unit lane that this lane checks */
-  for (int j = 0; j < 32; ++j) {
-    const unsigned long long bpi = __shfl_sync(0xffffffffu, (unsigned long long)p, j);
-    const uint32_t bsize = __shfl_sync(0xffffffffu, size, j);
-    const uint32_t bkey = __shfl_sync(0xffffffffu, key, j);
-    if (!bpi) continue;
-    unsigned char *bp = reinterpret_cast<unsigned char *>(bpi);
-    uint4 *u4 = reinterpret_cast<uint4 *>(bp);
-    const uint32_t nw = bsize >> 2, tail = bsize & 3, units = nw >> 2;
-    const unsigned rest_lane = units & 31;
+  if (!p) size = 0;
+  const unsigned rd = OP == PAY_FUSED ? (lane + 1) & 31 : lane;   /* lane whose units this lane checks */
+  const uint32_t units = size >> 4;
+  const bool flat = units <= pay_flat(OP);
+  if (OP & PAY_CHECK) a.words += (size >> 2) + ((size & 3) != 0);
+  if (__any_sync(FULL, (flat && units) || (size & 15))) {
+    const payload_acc r = payload_row<OP>(p, size, key, flat ? units : 0);
+    a.mism += r.mism;
+    a.x ^= r.x;
+    a.s += r.s;
+  }
+
+  /* the larger blocks, one at a time */
+  const unsigned long long pol = stream_policy();
+  for (unsigned big = __ballot_sync(FULL, !flat); big; big &= big - 1) {
+    const int j = __ffs(big) - 1;
+    uint4 *u4 = reinterpret_cast<uint4 *>(__shfl_sync(FULL, reinterpret_cast<unsigned long long>(p), j));
+    const uint32_t bu = __shfl_sync(FULL, units, j), bkey = __shfl_sync(FULL, key, j);
     if (OP & PAY_WRITE) {
 #pragma unroll 4
-      for (uint32_t u = lane; u < units; u += 32) u4[u] = pat4(bkey, 4 * u);
-      if (lane == rest_lane) block_rest<true>(bp, bkey, nw, tail, a);
+      for (uint32_t u = lane; u < bu; u += 32) st_stream(u4 + u, pat4(bkey, 4 * u), pol);
     }
     if (OP == PAY_FUSED) __syncwarp();
     if (OP & PAY_CHECK) {
       uint32_t u = rd;
-      for (; u + 96 < units; u += 128) {          /* four independent 16-byte loads in flight */
-        const uint4 g0 = __ldcg(u4 + u), g1 = __ldcg(u4 + u + 32), g2 = __ldcg(u4 + u + 64),
-                    g3 = __ldcg(u4 + u + 96);
+      for (; u + 96 < bu; u += 128) {          /* four independent 16-byte loads in flight */
+        const uint4 g0 = ld_stream(u4 + u, pol), g1 = ld_stream(u4 + u + 32, pol), g2 = ld_stream(u4 + u + 64, pol),
+                    g3 = ld_stream(u4 + u + 96, pol);
         check4(g0, pat4(bkey, 4 * u), a);
         check4(g1, pat4(bkey, 4 * (u + 32)), a);
         check4(g2, pat4(bkey, 4 * (u + 64)), a);
         check4(g3, pat4(bkey, 4 * (u + 96)), a);
       }
-      for (; u < units; u += 32) check4(__ldcg(u4 + u), pat4(bkey, 4 * u), a);
-      if (lane == (OP == PAY_FUSED ? (rest_lane + 31) & 31 : rest_lane)) {
-        block_rest<false>(bp, bkey, nw, tail, a);
-        a.words += nw + (tail != 0);
+      if (u + 32 < bu) {
+        const uint4 g0 = ld_stream(u4 + u, pol), g1 = ld_stream(u4 + u + 32, pol);
+        check4(g0, pat4(bkey, 4 * u), a);
+        check4(g1, pat4(bkey, 4 * (u + 32)), a);
+        u += 64;
       }
+      if (u < bu) check4(ld_stream(u4 + u, pol), pat4(bkey, 4 * u), a);
     }
   }
 }
 
-/* block reduction of the check counters into *out */
-__device__ inline void flush_acc(payload_acc &a, unsigned long long nulls, ouro_check *out) {
-  __shared__ unsigned long long sm[5];
+/* block reduction of the check counters into sm (shared memory); ends with a
+ * block barrier */
+__device__ inline void block_acc(payload_acc &a, unsigned long long nulls, unsigned long long (&sm)[5]) {
   if (threadIdx.x < 5) sm[threadIdx.x] = 0;
   __syncthreads();
   unsigned long long mism = a.mism;   /* per lane 32 bits; summed over the warp in 64 */
@@ -226,12 +347,54 @@ __device__ inline void flush_acc(payload_acc &a, unsigned long long nulls, ouro_
     atomicAdd(&sm[4], a.words);
   }
   __syncthreads();
+}
+
+/* the block's check counters added to *out (zero when the kernel began) */
+__device__ inline void flush_acc(payload_acc &a, unsigned long long nulls, ouro_check *out) {
+  __shared__ unsigned long long sm[5];
+  block_acc(a, nulls, sm);
   if (threadIdx.x == 0) {
     if (sm[0]) atomicAdd(&out->nulls, sm[0]);
     if (sm[1]) atomicAdd(&out->mismatches, sm[1]);
     atomicXor(&out->xor64, sm[2]);
     atomicAdd(&out->sum64, sm[3]);
     atomicAdd(&out->words, sm[4]);
+  }
+}
+
+/* One launch's work slot (a 128-byte line of the heap's metadata): all zero
+ * between launches.  The blocks add their counters to acc; the last one to
+ * finish writes the sums to *out and leaves the slot zero for the next
+ * launch, so a launch needs no memset of its counters or its result. */
+struct work_slot {
+  unsigned long long next;     /* requests handed out past the warps' first tasks */
+  unsigned long long acc[5];   /* nulls, mismatches, xor, sum, words */
+  unsigned long long done;     /* blocks finished */
+};
+__device__ inline void finish_acc(payload_acc &a, unsigned long long nulls, work_slot *w, ouro_check *out) {
+  __shared__ unsigned long long sm[5];
+  block_acc(a, nulls, sm);
+  if (threadIdx.x == 0) {
+    if (sm[0]) atomicAdd(&w->acc[0], sm[0]);
+    if (sm[1]) atomicAdd(&w->acc[1], sm[1]);
+    atomicXor(&w->acc[2], sm[2]);
+    atomicAdd(&w->acc[3], sm[3]);
+    atomicAdd(&w->acc[4], sm[4]);
+    __threadfence();
+    if (atomicAdd(&w->done, 1ull) == gridDim.x - 1) {
+      __threadfence();
+      unsigned long long *o = reinterpret_cast<unsigned long long *>(out);   /* five words, in acc's order */
+      unsigned long long r[5];
+#pragma unroll
+      for (int k = 0; k < 5; ++k) r[k] = ld_rlx(&w->acc[k]);
+#pragma unroll
+      for (int k = 0; k < 5; ++k) {
+        o[k] = r[k];
+        w->acc[k] = 0;
+      }
+      w->next = 0;
+      w->done = 0;
+    }
   }
 }
 
