@@ -349,13 +349,15 @@ ouro_status ouro_serve_per_launch(ouro_heap *h, const uint32_t *d_arrive_step, c
 size_t ouro_graph_vertex_bytes(void);
 /* Every vertex gets an empty list of 4 entries (16 B from the heap).
  * d_ctl (device, 4 words, cleared): [0] entries appended, [1] failed
- * mallocs, [2] entries skipped after a lock wait ran out. */
+ * mallocs, [2] entries skipped after a wait ran out. */
 ouro_status ouro_graph_init(ouro_heap *h, void *d_vertices, uint32_t n_vertices, unsigned long long *d_ctl,
                             void *stream);
 /* Append edge e's d_dst[e] to vertex d_src[e]'s list for all n_edges: a
  * list that is full doubles (malloc 2x, copy, free old) one step at a time
  * up to one chunk of entries, then grows by chained one-chunk overflow
- * segments.  Per-vertex locks, bounded. */
+ * segments.  Places at the end of a list are reserved with one atomic per
+ * block and source; every wait is bounded.  Insertions on several streams may
+ * run at the same time. */
 ouro_status ouro_graph_insert(ouro_heap *h, void *d_vertices, const uint32_t *d_src, const uint32_t *d_dst,
                               uint64_t n_edges, unsigned long long *d_ctl, void *stream);
 /* Copy every vertex's entries to d_out[d_offsets[v] ..] (offsets = prefix
