@@ -401,7 +401,7 @@ def measure_serving(variants=(("page_array", "persistent"), ("page_array", "per_
     """Serving: 64 GiB heap of 16 KiB blocks; Poisson session arrivals
     (2000/s, 10 ms steps); lognormal session sizes (median 4 MiB, sigma 1);
     one block per session per step; admission up to 95 % of the blocks;
-    `steps` steps in one cooperative kernel (persistent) or four plain
+    `steps` steps in one cooperative kernel (persistent) or two plain
     launches per step (per_launch).  Verified against the oracle's admission
     schedule and per-session checksums (64 sampled completed sessions)."""
     import numpy as np
@@ -721,7 +721,7 @@ def main():
 def added_patterns() -> dict:
     """The three added usage patterns at their full sizes, each verified:
     batching (every form; fused / graph / persistent against four launches
-    per batch), serving (one cooperative loop against four launches per
+    per batch), serving (one cooperative loop against two launches per
     step; p50 / p99 step latency) and graph growth."""
     out = {}
     bt = measure_batching("page_array")

@@ -309,10 +309,11 @@ ouro_status ouro_batch_graph_destroy(ouro_batch_graph *g);
  *   d_slot_session n_slots ints, d_slot_k n_slots, d_slot_acc 3*n_slots,
  *   d_tables n_slots*max_blocks pointers, d_sess_out 5*n_sessions words
  *   (xor, sum, mismatches, admit step, done step; all ones if never),
- *   d_step_ns 3*`steps` %globaltimer stamps (after admission, growth and
- *   completion of each step), d_ctl 11 words (barrier state, next
- *   arrival, committed blocks, error flag, mallocs, frees, failed mallocs,
- *   free-slot stack top, sessions finished in the step, one reserved),
+ *   d_step_ns 3*`steps` %globaltimer stamps (each step's growth begins, has
+ *   ended, and its frees and the next step's admission have ended), d_ctl 11
+ *   words (barrier state, next arrival, committed blocks, error flag, mallocs,
+ *   frees, failed mallocs, free-slot stack top, sessions finished in even and
+ *   in odd steps),
  *   d_free_stack 2*n_slots slot ids (the free-slot stack, then the step's
  *   list of finished sessions, whose blocks are freed in tasks of 32 dealt
  *   to the warps in turn).
@@ -329,8 +330,8 @@ ouro_status ouro_serve(ouro_heap *h, const uint32_t *d_arrive_step, const uint32
                        void *stream);
 
 /* The same loop as plain per-launch kernels: for every step, one launch each
- * for admission, growth, completion and freeing, enqueued on `stream` in
- * order without a host wait (4 * steps + 2 launches).  Kernel boundaries
+ * for growth and for freeing with the next step's admission, enqueued on
+ * `stream` in order without a host wait (2 * steps + 3 launches).  Kernel boundaries
  * take the place of the grid barriers, so no cooperative launch is needed
  * and no wait can run out.  Arguments, buffers and results are those of
  * ouro_serve and equal its results for the same inputs; d_step_ns stamps

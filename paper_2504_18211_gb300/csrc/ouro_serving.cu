@@ -2,23 +2,22 @@
  * Serving: a request loop that stays on the device (one cooperative,
  * persistent kernel for all steps) over sessions whose memory grows.
  *
- * Each step:
- *   1. admission (block 0, warp 0): sessions that have arrived are admitted
- *      in arrival order while a session slot is free and the blocks committed
- *      to admitted sessions, plus the newcomer's total, stay within the
- *      admission cap (95 % of the heap's blocks); the warp weighs 32
- *      arrivals at a time and admits the longest run of them, from the
- *      first, that passes;
- *   2. growth (all warps): every active session allocates one block with
- *      ouro_malloc, records it in its block table, writes its pattern
- *      (seed + session id, block index) and reads it back through L2,
- *      folding the words into the session checksum;
- *   3. completion: a session that reached its size reports its checksum and
- *      its slot is free for the next step (one thread per slot); after a
- *      barrier, the finished sessions' blocks are cut into tasks of 32 (one
- *      round of a warp) dealt to the warps in turn, so that the step's
- *      frees spread over the grid and one long session does not hold the
- *      step for a single warp.
+ * Each step has two phases, with a grid barrier after each:
+ *   1. growth (all blocks): every active session allocates one block with
+ *      ouro_malloc, records it in its block table, writes its pattern (seed +
+ *      session id, block index) and reads it back through L2, folding the
+ *      words into the session checksum; a session that has reached its size
+ *      reports its checksum, gives its slot back and is listed;
+ *   2. freeing and admission: the listed sessions' blocks are cut into tasks
+ *      of 32 (one round of a warp) dealt to the warps in turn, so that the
+ *      step's frees spread over the grid and one long session does not hold
+ *      the step for a single warp.  Meanwhile the grid's last warp admits the
+ *      sessions of the next step, in arrival order, while a session slot is
+ *      free and the blocks committed to admitted sessions, plus the
+ *      newcomer's total, stay within the admission cap (95 % of the heap's
+ *      blocks); it weighs 32 arrivals at a time and admits the longest run of
+ *      them, from the first, that passes.  Admission needs slots and
+ *      committed blocks, which phase 1 settled, and nothing that is freed.
  * The allocator state, the session table and the block tables stay resident
  * for the whole run; requests that arrive while others are running are
  * admitted as slots and memory free up, and their work overlaps on the GPU.
@@ -47,7 +46,7 @@ struct serve_args {
   uint32_t n_sessions;
   /* slots */
   uint32_t n_slots, max_blocks;
-  int *slot_session;             /* session id or -1 */
+  int *slot_session;             /* session id, -1 free, -2 - id: admitted, no block yet */
   uint32_t *slot_k;              /* blocks allocated so far */
   unsigned long long *slot_acc;  /* per slot: xor, sum, mismatches */
   unsigned long long *tables;    /* n_slots x max_blocks block pointers */
@@ -56,8 +55,7 @@ struct serve_args {
   unsigned long long *step_ns;   /* per step: %globaltimer after admission, growth and completion (3 words) */
   unsigned long long *ctl;       /* [0] barrier count, [1] barrier generation, [2] next arrival,
                                     [3] committed blocks, [4] error, [5] mallocs, [6] frees, [7] failed,
-                                    [8] free-slot stack top, [9] sessions finished this step,
-                                    [10] reserved */
+                                    [8] free-slot stack top, [9 + step % 2] sessions finished this step */
   uint32_t *free_stack;          /* free slot ids (stack of n_slots) */
   uint32_t *done_list;           /* slots whose sessions finished this step (n_slots) */
   uint32_t steps;
@@ -93,36 +91,13 @@ __device__ bool grid_barrier(unsigned long long *ctl, unsigned nblocks, unsigned
           ok = 0;
           break;
         }
-        __nanosleep(128);
+        __nanosleep(32);
       }
     }
     if (ld_acq(&ctl[4])) ok = 0;
   }
   __syncthreads();
   return ok != 0;
-}
-
-/* Pattern of one block, written and read back by the whole warp; the
- * block's folded checksum lands in (x, s, mism) of every lane. */
-__device__ void serve_block_payload(unsigned char *bp, uint32_t bytes, uint32_t key, unsigned long long &x,
-                                    unsigned long long &s, unsigned long long &mism) {
-  const unsigned lane = laneid();
-  uint4 *u4 = reinterpret_cast<uint4 *>(bp);
-  const uint32_t units = bytes >> 4;
-#pragma unroll 4
-  for (uint32_t u = lane; u < units; u += 32) u4[u] = pat4(key, 4 * u);
-  __syncwarp();
-  payload_acc a;
-  for (uint32_t u = (lane + 1) & 31; u < units; u += 32) check4(__ldcg(u4 + u), pat4(key, 4 * u), a);
-  unsigned long long m = a.mism;
-  for (int o = 16; o; o >>= 1) {
-    a.x ^= __shfl_xor_sync(0xffffffffu, a.x, o);
-    a.s += __shfl_xor_sync(0xffffffffu, a.s, o);
-    m += __shfl_xor_sync(0xffffffffu, m, o);
-  }
-  x = a.x;
-  s = a.s;
-  mism = m;
 }
 
 /* ---------------------------------------------------------------- phases
@@ -137,13 +112,15 @@ __device__ void serve_init(const serve_args &A) {
   if (blockIdx.x == 0 && threadIdx.x == 0) A.ctl[8] = A.n_slots;
 }
 
-/* 1. admission (warp 0 of block 0): arrival order, a free slot (stack),
- *    committed + newcomer <= cap */
+/* Admission for step `step` (the grid's last warp, the last to get freeing
+ * tasks): arrival order, a free slot (stack), committed + newcomer <= cap.
+ * Also empties the finished count that the step will use. */
 __device__ void serve_admit(const serve_args &A, uint32_t step) {
-  if (blockIdx.x != 0 || threadIdx.x >= 32) return;
+  if (blockIdx.x != gridDim.x - 1 || threadIdx.x < blockDim.x - 32) return;
   const unsigned lane = laneid();
-  if (lane == 0) A.ctl[9] = 0;       /* the previous step's frees are all done */
-  unsigned long long next = A.ctl[2], committed = A.ctl[3], top = A.ctl[8];
+  if (lane == 0) A.ctl[9 + (step & 1)] = 0;
+  unsigned long long next = A.ctl[2], committed = *(volatile unsigned long long *)&A.ctl[3],
+                     top = *(volatile unsigned long long *)&A.ctl[8];
   for (;;) {
     const unsigned long long i = next + lane;
     const bool arrived = i < A.n_sessions && A.arrive_step[i] <= step;
@@ -156,10 +133,8 @@ __device__ void serve_admit(const serve_args &A, uint32_t step) {
     const unsigned okm = __ballot_sync(0xffffffffu, ok);
     const unsigned n_adm = okm == 0xffffffffu ? 32u : (unsigned)(__ffs(~okm) - 1);   /* leading run */
     if (lane < n_adm) {
-      const uint32_t slot = A.free_stack[top - 1 - lane];
-      A.slot_session[slot] = (int)i;
-      A.slot_k[slot] = 0;
-      A.slot_acc[3 * slot] = A.slot_acc[3 * slot + 1] = A.slot_acc[3 * slot + 2] = 0;
+      const uint32_t slot = __ldcg(&A.free_stack[top - 1 - lane]);
+      A.slot_session[slot] = -2 - (int)i;
       A.sess_out[5 * i + 3] = step;
     }
     if (n_adm) committed += __shfl_sync(0xffffffffu, cum, n_adm - 1);
@@ -175,60 +150,128 @@ __device__ void serve_admit(const serve_args &A, uint32_t step) {
   __threadfence();
 }
 
-/* 2. growth: one session per warp: lane 0 allocates, the warp writes and
- *    reads back the block */
+/* Growth and completion.  Block b of the grid holds slots b, b + grid, ...,
+ * up to 32 of them at a time: its first warp reads their sessions, a lane
+ * each, and allocates all their blocks with one queue operation; then the
+ * block's warps write the new blocks in pieces of SERVE_PIECE units, all of
+ * them, and read them back, each warp what its neighbour wrote, eight loads
+ * in flight per lane.  One warp per session had walked the allocator's chain
+ * and 16 KiB alone, sessions one after another.  What is left is a chain of
+ * L2 round trips, not bandwidth: 400 steps of about 1700 blocks of 16 KiB took
+ * 12.3 ms with five barriers and phases a step, 8.0 ms so (28 MB a step would
+ * take 4.2 us of its 20 at the copy rate). */
+constexpr uint32_t SERVE_PIECE = 256;
+
 template <int V>
-__device__ void serve_grow(const serve_args &A) {
-  const unsigned lane = laneid();
-  const unsigned warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const unsigned nwarps = (gridDim.x * blockDim.x) >> 5;
+__device__ void serve_grow(const serve_args &A, uint32_t step) {
+  __shared__ unsigned char *s_bp[32];
+  __shared__ uint32_t s_key[32];
+  __shared__ unsigned long long s_sum[32];
+  __shared__ unsigned s_xor[32], s_mism[32];
+  __shared__ unsigned s_n;
+  const unsigned lane = laneid(), warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
   const ouro_heap_dev &h = A.h;
-  for (uint32_t slot = warp; slot < A.n_slots; slot += nwarps) {
-    const int sess = A.slot_session[slot];
-    if (sess < 0) continue;
-    const uint32_t k = A.slot_k[slot];
-    if (k >= A.blocks[sess]) continue;
-    /* lane 0 asks; the other 31 lanes help the warp's carves */
-    /* (a step's growth can carve thousands of chunks: eight slot writes per
-     *  lane in flight while the warp fills them) */
-    unsigned long long bp = reinterpret_cast<unsigned long long>(malloc_v<V, 8>(h, A.block_bytes, lane == 0));
-    if (lane == 0) {
-      if (bp) {
-        A.tables[(size_t)slot * A.max_blocks + k] = bp;
-        A.slot_k[slot] = k + 1;
-        atomicAdd(&A.ctl[5], 1ull);
-      } else {
-        atomicAdd(&A.ctl[7], 1ull);
+  const uint32_t units = A.block_bytes >> 4, per = (units + SERVE_PIECE - 1) / SERVE_PIECE;
+  for (unsigned long long first = blockIdx.x; first < A.n_slots; first += 32ull * gridDim.x) {
+    int sess = -1;
+    uint32_t k = 0, total = 0;
+    unsigned long long slot = 0, x = 0, sum = 0, mism = 0;
+    bool fresh = false, grown = false;
+    unsigned at = 0;
+    if (warp == 0) {
+      slot = first + (unsigned long long)lane * gridDim.x;
+      if (slot < A.n_slots) sess = __ldcg(&A.slot_session[slot]);
+      fresh = sess < -1;
+      if (fresh) sess = -2 - sess;
+      if (sess >= 0) {
+        total = A.blocks[sess];
+        if (!fresh) {
+          k = A.slot_k[slot];
+          x = A.slot_acc[3 * slot];
+          sum = A.slot_acc[3 * slot + 1];
+          mism = A.slot_acc[3 * slot + 2];
+        }
+      }
+      __syncwarp();
+      /* (a step's growth can carve thousands of chunks: eight slot writes per
+       *  lane in flight while the warp fills them) */
+      const bool want = sess >= 0 && k < total;
+      unsigned char *bp = static_cast<unsigned char *>(malloc_v<V, 8>(h, A.block_bytes, want));
+      __syncwarp();
+      grown = want && bp;
+      const unsigned gm = __ballot_sync(0xffffffffu, grown), wm = __ballot_sync(0xffffffffu, want);
+      at = __popc(gm & lanemask_lt());
+      if (grown) {
+        A.tables[slot * A.max_blocks + k] = reinterpret_cast<unsigned long long>(bp);
+        s_bp[at] = bp;
+        s_key[at] = fmix32((A.seed + (uint32_t)sess) ^ (k * OURO_GOLD));
+        s_sum[at] = 0;
+        s_xor[at] = s_mism[at] = 0;
+      }
+      if (lane == 0) {
+        s_n = __popc(gm);
+        if (gm) atomicAdd(&A.ctl[5], (unsigned long long)__popc(gm));
+        if (wm != gm) atomicAdd(&A.ctl[7], (unsigned long long)__popc(wm & ~gm));
       }
     }
-    bp = __shfl_sync(0xffffffffu, bp, 0);
-    if (!bp) continue;
-    const uint32_t key = fmix32((A.seed + (uint32_t)sess) ^ (k * OURO_GOLD));
-    unsigned long long x, sum, mism;
-    serve_block_payload(reinterpret_cast<unsigned char *>(bp), A.block_bytes, key, x, sum, mism);
-    if (lane == 0) {
-      A.slot_acc[3 * slot] ^= x;
-      A.slot_acc[3 * slot + 1] += sum;
-      A.slot_acc[3 * slot + 2] += mism;
+    __syncthreads();
+    const unsigned pieces = s_n * per;
+    const unsigned long long pol = stream_policy();
+    for (unsigned t = warp; t < pieces; t += nwarps) {
+      const unsigned b = t / per, u0 = (t - b * per) * SERVE_PIECE;
+      uint4 *u4 = reinterpret_cast<uint4 *>(s_bp[b]);
+      const uint32_t key = s_key[b], end = min(units, u0 + SERVE_PIECE);
+#pragma unroll 8
+      for (uint32_t u = u0 + lane; u < end; u += 32) st_stream(u4 + u, pat4(key, 4 * u), pol);
     }
-  }
-}
-
-/* 3a. completion: a session that reached its size reports, releases its
- *     slot (reused from the next step on) and is listed for freeing */
-__device__ void serve_complete(const serve_args &A, uint32_t step) {
-  for (uint32_t slot = blockIdx.x * blockDim.x + threadIdx.x; slot < A.n_slots; slot += gridDim.x * blockDim.x) {
-    const int sess = A.slot_session[slot];
-    if (sess < 0 || A.slot_k[slot] < A.blocks[sess]) continue;
-    A.sess_out[5 * sess + 0] = A.slot_acc[3 * slot];
-    A.sess_out[5 * sess + 1] = A.slot_acc[3 * slot + 1];
-    A.sess_out[5 * sess + 2] = A.slot_acc[3 * slot + 2];
-    A.sess_out[5 * sess + 4] = step;
-    atomicAdd(&A.ctl[6], (unsigned long long)A.slot_k[slot]);
-    atomicAdd(&A.ctl[3], 0ull - (unsigned long long)A.blocks[sess]);
-    A.slot_session[slot] = -1;
-    A.free_stack[atomicAdd(&A.ctl[8], 1ull)] = slot;
-    A.done_list[atomicAdd(&A.ctl[9], 1ull)] = slot;
+    __syncthreads();
+    for (unsigned t = (warp + 1) % nwarps; t < pieces; t += nwarps) {
+      const unsigned b = t / per, u0 = (t - b * per) * SERVE_PIECE;
+      const uint4 *u4 = reinterpret_cast<const uint4 *>(s_bp[b]);
+      const uint32_t key = s_key[b], end = min(units, u0 + SERVE_PIECE);
+      payload_acc a;
+      uint4 g[SERVE_PIECE / 32];
+#pragma unroll
+      for (unsigned r = 0; r < SERVE_PIECE / 32; ++r)
+        if (u0 + 32 * r + lane < end) g[r] = ld_stream(u4 + u0 + 32 * r + lane, pol);
+#pragma unroll
+      for (unsigned r = 0; r < SERVE_PIECE / 32; ++r)
+        if (u0 + 32 * r + lane < end) check4(g[r], pat4(key, 4 * (u0 + 32 * r + lane)), a);
+      const unsigned ax = __reduce_xor_sync(0xffffffffu, a.x), am = __reduce_add_sync(0xffffffffu, a.mism);
+      for (int o = 16; o; o >>= 1) a.s += __shfl_xor_sync(0xffffffffu, a.s, o);
+      if (lane == 0) {
+        atomicXor(&s_xor[b], ax);
+        atomicAdd(&s_sum[b], a.s);
+        if (am) atomicAdd(&s_mism[b], am);
+      }
+    }
+    __syncthreads();
+    if (warp == 0 && sess >= 0) {
+      if (grown) {
+        ++k;
+        x ^= s_xor[at];
+        sum += s_sum[at];
+        mism += s_mism[at];
+      }
+      A.slot_k[slot] = k;
+      if (k < total) {
+        if (fresh) A.slot_session[slot] = sess;
+        A.slot_acc[3 * slot] = x;
+        A.slot_acc[3 * slot + 1] = sum;
+        A.slot_acc[3 * slot + 2] = mism;
+      } else {   /* complete: report, release the slot (reused from the next step on), list it for freeing */
+        A.sess_out[5ull * sess + 0] = x;
+        A.sess_out[5ull * sess + 1] = sum;
+        A.sess_out[5ull * sess + 2] = mism;
+        A.sess_out[5ull * sess + 4] = step;
+        atomicAdd(&A.ctl[6], (unsigned long long)k);
+        atomicAdd(&A.ctl[3], 0ull - (unsigned long long)total);
+        A.slot_session[slot] = -1;
+        A.free_stack[atomicAdd(&A.ctl[8], 1ull)] = (uint32_t)slot;
+        A.done_list[atomicAdd(&A.ctl[9 + (step & 1)], 1ull)] = (uint32_t)slot;
+      }
+    }
+    __syncthreads();
   }
 }
 
@@ -236,25 +279,25 @@ __device__ void serve_complete(const serve_args &A, uint32_t step) {
  * step's frees spread over as many warps as there are rounds of work */
 constexpr uint32_t SERVE_FREE_TASK = 32;
 
-/* 3b. the listed sessions' blocks, in tasks of SERVE_FREE_TASK blocks; warp
+/* Freeing: the listed sessions' blocks, in tasks of SERVE_FREE_TASK blocks; warp
  *     w takes tasks w, w + nwarps, ... (tasks are of equal size, so a static
  *     share balances without a shared counter): task c is piece
  *     c - (pieces of the earlier list entries) of the first entry whose
  *     running piece count passes c */
 template <int V>
-__device__ void serve_free(const serve_args &A) {
+__device__ void serve_free(const serve_args &A, uint32_t step) {
   const unsigned lane = laneid();
   const unsigned long long nwarps = (gridDim.x * blockDim.x) >> 5;
   const ouro_heap_dev &h = A.h;
-  const unsigned long long nl = *(volatile unsigned long long *)&A.ctl[9];
+  const unsigned long long nl = *(volatile unsigned long long *)&A.ctl[9 + (step & 1)];
   for (unsigned long long c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;; c += nwarps) {
     unsigned long long before = 0;
     uint32_t slot = 0, nb = 0;
     bool found = false;
     for (unsigned long long i0 = 0; i0 < nl && !found; i0 += 32) {
       const unsigned long long i = i0 + lane;
-      const uint32_t s_i = i < nl ? A.done_list[i] : 0;
-      const uint32_t nb_i = i < nl ? A.slot_k[s_i] : 0;
+      const uint32_t s_i = i < nl ? __ldcg(&A.done_list[i]) : 0;
+      const uint32_t nb_i = i < nl ? __ldcg(&A.slot_k[s_i]) : 0;
       unsigned long long pc = (nb_i + SERVE_FREE_TASK - 1) / SERVE_FREE_TASK, incl = pc;
       for (int o = 1; o < 32; o <<= 1) {
         const unsigned long long y = __shfl_up_sync(0xffffffffu, incl, o);
@@ -275,7 +318,7 @@ __device__ void serve_free(const serve_args &A) {
     const uint32_t b_lo = (uint32_t)(c - before) * SERVE_FREE_TASK, b_hi = min(nb, b_lo + SERVE_FREE_TASK);
     for (uint32_t b0 = b_lo; b0 < b_hi; b0 += 32) {
       const uint32_t b = b0 + lane;
-      void *p = b < b_hi ? reinterpret_cast<void *>(A.tables[(size_t)slot * A.max_blocks + b]) : nullptr;
+      void *p = b < b_hi ? reinterpret_cast<void *>(__ldcg(&A.tables[(size_t)slot * A.max_blocks + b])) : nullptr;
       if (b < b_hi) free_v<V>(h, p);
       __syncwarp();
     }
@@ -283,39 +326,47 @@ __device__ void serve_free(const serve_args &A) {
 }
 
 /* The cooperative form: every step in one launch, phases separated by grid
- * barriers; block 0 stamps %globaltimer after admission, growth and freeing. */
+ * barriers; block 0 stamps %globaltimer when a step begins to grow, when it
+ * has grown and when its frees and the next admission are done. */
 template <int V>
-__global__ void __launch_bounds__(256) k_serve(serve_args A) {
+__global__ void __launch_bounds__(256, 2) k_serve(serve_args A) {
   serve_init(A);
   if (!grid_barrier(A.ctl, gridDim.x, A.spin_limit)) return;
+  if (A.steps) serve_admit(A, 0);
+  if (!grid_barrier(A.ctl, gridDim.x, A.spin_limit)) return;
+  const bool stamps = blockIdx.x == 0 && threadIdx.x == 0;
   for (uint32_t step = 0; step < A.steps; ++step) {
-    serve_admit(A, step);
+    if (stamps) A.step_ns[3 * step] = globaltimer();
+    serve_grow<V>(A, step);
     if (!grid_barrier(A.ctl, gridDim.x, A.spin_limit)) return;
-    if (blockIdx.x == 0 && threadIdx.x == 0) A.step_ns[3 * step] = globaltimer();
-    serve_grow<V>(A);
+    if (stamps) A.step_ns[3 * step + 1] = globaltimer();
+    if (step + 1 < A.steps) serve_admit(A, step + 1);
+    serve_free<V>(A, step);
     if (!grid_barrier(A.ctl, gridDim.x, A.spin_limit)) return;
-    if (blockIdx.x == 0 && threadIdx.x == 0) A.step_ns[3 * step + 1] = globaltimer();
-    serve_complete(A, step);
-    if (!grid_barrier(A.ctl, gridDim.x, A.spin_limit)) return;
-    serve_free<V>(A);
-    if (!grid_barrier(A.ctl, gridDim.x, A.spin_limit)) return;
-    if (blockIdx.x == 0 && threadIdx.x == 0) A.step_ns[3 * step + 2] = globaltimer();
+    if (stamps) A.step_ns[3 * step + 2] = globaltimer();
   }
 }
 
 /* The per-launch form: one kernel per phase and step, in stream order.  A
- * phase kernel first stamps %globaltimer into step_ns[stamp] (stamp >= 0):
- * the moment the previous phase had finished on the whole grid. */
-enum { PH_INIT, PH_ADMIT, PH_GROW, PH_COMPLETE, PH_FREE, PH_STAMP };
+ * phase kernel first stamps %globaltimer into step_ns[stamp] and, where
+ * stamp2 >= 0, step_ns[stamp2]: the moment the previous phase had finished on
+ * the whole grid. */
+enum { PH_INIT, PH_ADMIT, PH_GROW, PH_FREE, PH_STAMP };
 
 template <int V, int PH>
-__global__ void __launch_bounds__(256) k_serve_phase(serve_args A, uint32_t step, int stamp) {
-  if (stamp >= 0 && blockIdx.x == 0 && threadIdx.x == 0) A.step_ns[stamp] = globaltimer();
+__global__ void __launch_bounds__(256, 2) k_serve_phase(serve_args A, uint32_t step, int stamp, int stamp2) {
+  if (blockIdx.x == 0 && threadIdx.x == 0 && stamp >= 0) {
+    const unsigned long long t = globaltimer();
+    A.step_ns[stamp] = t;
+    if (stamp2 >= 0) A.step_ns[stamp2] = t;
+  }
   if (PH == PH_INIT) serve_init(A);
   if (PH == PH_ADMIT) serve_admit(A, step);
-  if (PH == PH_GROW) serve_grow<V>(A);
-  if (PH == PH_COMPLETE) serve_complete(A, step);
-  if (PH == PH_FREE) serve_free<V>(A);
+  if (PH == PH_GROW) serve_grow<V>(A, step);
+  if (PH == PH_FREE) {
+    if (step + 1 < A.steps) serve_admit(A, step + 1);
+    serve_free<V>(A, step);
+  }
 }
 
 #if OURO_SHARD_ENTRIES
@@ -342,8 +393,9 @@ ouro_status serve(const void *args, int blocks_per_sm, cudaStream_t s) {
   return OURO_OK;
 }
 
-/* the per-launch form: four launches per step (admission, growth,
- * completion, freeing) plus the set-up and a final stamp, in stream order */
+/* the per-launch form: two launches per step (growth; freeing and the next
+ * admission) plus the set-up, the first admission and a final stamp, in
+ * stream order */
 template <int V>
 ouro_status serve_steps(const void *args, int blocks_per_sm, cudaStream_t s) {
   const serve_args &A = *static_cast<const serve_args *>(args);
@@ -355,26 +407,23 @@ ouro_status serve_steps(const void *args, int blocks_per_sm, cudaStream_t s) {
     grow_sm = std::min(grow_sm, blocks_per_sm);
     free_sm = std::min(free_sm, blocks_per_sm);
   }
-  /* growth: a warp per slot at most; slots: a thread per slot */
-  const unsigned grow_g = (unsigned)std::max(1, std::min(grow_sm * sms, (int)((A.n_slots + 7) / 8)));
+  /* growth: a block per slot at most; slots: a thread per slot */
+  const unsigned grow_g = (unsigned)std::max(1, (int)std::min<long long>((long long)grow_sm * sms, A.n_slots));
   const unsigned free_g = (unsigned)std::max(1, free_sm * sms);
   const unsigned slot_g = (unsigned)std::max(1u, std::min((A.n_slots + 255) / 256, 8u * sms));
-  k_serve_phase<V, PH_INIT><<<slot_g, 256, 0, s>>>(A, 0, -1);
+  k_serve_phase<V, PH_INIT><<<slot_g, 256, 0, s>>>(A, 0, -1, -1);
+  OURO_LAUNCHED();
+  if (!A.steps) return OURO_OK;
+  k_serve_phase<V, PH_ADMIT><<<1, 32, 0, s>>>(A, 0, -1, -1);
   OURO_LAUNCHED();
   for (uint32_t step = 0; step < A.steps; ++step) {
-    k_serve_phase<V, PH_ADMIT><<<1, 32, 0, s>>>(A, step, step ? (int)(3 * step - 1) : -1);
+    k_serve_phase<V, PH_GROW><<<grow_g, 256, 0, s>>>(A, step, (int)(3 * step), step ? (int)(3 * step - 1) : -1);
     OURO_LAUNCHED();
-    k_serve_phase<V, PH_GROW><<<grow_g, 256, 0, s>>>(A, step, (int)(3 * step));
-    OURO_LAUNCHED();
-    k_serve_phase<V, PH_COMPLETE><<<slot_g, 256, 0, s>>>(A, step, (int)(3 * step + 1));
-    OURO_LAUNCHED();
-    k_serve_phase<V, PH_FREE><<<free_g, 256, 0, s>>>(A, step, -1);
+    k_serve_phase<V, PH_FREE><<<free_g, 256, 0, s>>>(A, step, (int)(3 * step + 1), -1);
     OURO_LAUNCHED();
   }
-  if (A.steps) {
-    k_serve_phase<V, PH_STAMP><<<1, 32, 0, s>>>(A, 0, (int)(3 * A.steps - 1));
-    OURO_LAUNCHED();
-  }
+  k_serve_phase<V, PH_STAMP><<<1, 32, 0, s>>>(A, 0, (int)(3 * A.steps - 1), -1);
+  OURO_LAUNCHED();
   return OURO_OK;
 }
 

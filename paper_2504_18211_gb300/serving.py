@@ -37,7 +37,7 @@ class ServeRun:
     def run(self, heap, cap_blocks: int, blocks_per_sm: int = 0, form: str = "persistent") -> float:
         """One call of the loop; returns its duration in ms (CUDA events).
         form "persistent": ouro_serve, every step in one cooperative kernel;
-        "per_launch": ouro_serve_per_launch, four launches per step."""
+        "per_launch": ouro_serve_per_launch, two launches per step."""
         torch = self.torch
         if form not in ("persistent", "per_launch"):
             raise ValueError(f"unknown serving form {form!r}")
