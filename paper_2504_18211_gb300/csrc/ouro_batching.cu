@@ -24,50 +24,74 @@ using namespace ouro::detail;
 
 namespace {
 
-constexpr unsigned TASK_REQ = 256;   /* requests per persistent task: 8 warp iterations */
+constexpr unsigned TASK_REQ_LOG = 8;   /* 256 requests per persistent task (the offsets' unit, see ouro.h) */
 
+/* Warps claim work in rounds of 2^round_log requests: 32, or fewer on a pass
+ * too short to give every resident warp a round of 32.  Round r of the launch
+ * is round r mod R of task r / R, R = 256 >> round_log (a batch's last
+ * task may have empty rounds).  A claim is a whole task until `last_wave`,
+ * then one round: with whole tasks to the end a warp had 4 or 5 of them on a
+ * pass of 6 M requests, and the kernel ended with the fives (96 batches of up
+ * to 2^18 requests, staged: 3.22 ms, 3.05 so). */
 template <int V, bool STAGE>
 __global__ void __launch_bounds__(256, ouro_page_queues(V) ? 4 : 2)   /* chunk queues: no spills at 2 per SM */
 k_batches_persistent(ouro_heap_dev h, const uint32_t *sizes, const unsigned long long *offs,
                      const unsigned long long *task_offs, unsigned n_batches, uint32_t seed, int mode,
-                     ouro_check *out, unsigned long long *work, unsigned long long n_tasks) {
+                     ouro_check *out, unsigned long long *work, unsigned long long n_rounds,
+                     unsigned long long last_wave, unsigned round_log) {
   __shared__ ouro_block_ctx<8> ctx;
   if (STAGE) ouro_block_begin(ctx);
-  const unsigned lane = laneid();
+  const unsigned lane = laneid(), rpt_log = TASK_REQ_LOG - round_log;   /* rounds per task */
+  payload_acc a;
+  unsigned long long nulls = 0, next = 0, end = 0;
+  unsigned b = 0;
+  bool any = false;                        /* a holds counts of batch b */
+  unsigned long long task_lo = 0, task_hi = 0, base = 0, count = 0;   /* tasks, requests of batch b */
   for (;;) {
-    unsigned long long task = 0;
-    if (lane == 0) task = atomicAdd(work, 1ull);
-    task = __shfl_sync(0xffffffffu, task, 0);
-    if (task >= n_tasks) break;
-    unsigned lo = 0, hi = n_batches;       /* task_offs[lo] <= task < task_offs[hi] */
-    while (hi - lo > 1) {
-      const unsigned mid = (lo + hi) >> 1;
-      if (task_offs[mid] <= task) lo = mid;
-      else hi = mid;
+    if (next == end) {
+      const unsigned take = end < last_wave ? 1u << rpt_log : 1u;
+      if (lane == 0) next = atomicAdd(work, (unsigned long long)take);
+      next = __shfl_sync(0xffffffffu, next, 0);
+      if (next >= n_rounds) break;
+      end = next + take;
     }
-    const unsigned b = lo;
-    const unsigned long long base = offs[b], count = offs[b + 1] - offs[b];
-    const unsigned long long local0 = (task - task_offs[b]) * TASK_REQ;
-    payload_acc a;
-    unsigned long long nulls = 0;
-    for (unsigned r = 0; r < TASK_REQ / 32; ++r) {
-      const unsigned long long i = local0 + r * 32 + lane;
-      const bool active = i < count;
-      if (!__any_sync(0xffffffffu, active)) break;
-      const uint32_t sz = active ? sizes[base + i] : 0;
-      unsigned char *p = nullptr;
-      if (STAGE) p = static_cast<unsigned char *>(stage_malloc_v<V>(ctx, h, sz, active));
-      else if (active) p = static_cast<unsigned char *>(malloc_v<V>(h, sz));
-      if (active && !p) nulls++;
-      __syncwarp();
-      warp_payload<PAY_FUSED>(p, sz, (uint32_t)i, seed + b, mode, a);
-      __syncwarp();
-      if (STAGE) stage_free_v<V>(ctx, h, p);
-      else if (active) free_v<V>(h, p);
-      __syncwarp();
+    const unsigned long long task = next >> rpt_log;
+    if (task < task_lo || task >= task_hi) {
+      if (next >= n_rounds) break;
+      if (any) warp_flush(a, nulls, &out[b]);
+      a = payload_acc();
+      nulls = 0;
+      any = false;
+      unsigned lo = 0, hi = n_batches;       /* task_offs[lo] <= task < task_offs[hi] */
+      while (hi - lo > 1) {
+        const unsigned mid = (lo + hi) >> 1;
+        if (task_offs[mid] <= task) lo = mid;
+        else hi = mid;
+      }
+      b = lo;
+      task_lo = task_offs[b];
+      task_hi = task_offs[b + 1];
+      base = offs[b];
+      count = offs[b + 1] - base;
     }
-    warp_flush(a, nulls, &out[b]);
+    const unsigned long long i = ((next - (task_lo << rpt_log)) << round_log) + lane;
+    ++next;
+    const bool active = lane >> round_log == 0 && i < count;
+    if (!__any_sync(0xffffffffu, active)) continue;
+    any = true;
+    const uint32_t sz = active ? sizes[base + i] : 0;
+    unsigned char *p = nullptr;
+    if (STAGE) p = static_cast<unsigned char *>(stage_malloc_v<V>(ctx, h, sz, active));
+    else p = static_cast<unsigned char *>(malloc_v<V>(h, sz, active));
+    if (active && !p) nulls++;
+    __syncwarp();
+    warp_payload<PAY_FUSED>(p, sz, (uint32_t)i, seed + b, mode, a);
+    __syncwarp();
+    if (STAGE) ouro::detail::stage_free<V, 8>(ctx, h, p, __activemask(), p ? size_class(h, sz) : -1);
+    else free_v<V>(h, p);
+    __syncwarp();
   }
+  if (any) warp_flush(a, nulls, &out[b]);
   if (STAGE) ouro_block_end_v<V>(ctx, h);
 }
 
@@ -89,22 +113,31 @@ int persistent_blocks_per_sm(int blocks_per_sm) {
   return per_sm;
 }
 
+template <int V, bool STAGE>
+ouro_status batches_form(ouro_heap *H, const uint32_t *d_sizes, const unsigned long long *d_offs,
+                         const unsigned long long *d_task_offs, uint32_t n_batches, uint64_t n_tasks, uint32_t seed,
+                         int mode, ouro_check *d_out, unsigned long long *d_work, int blocks_per_sm, cudaStream_t s) {
+  const int grid = std::max(1, persistent_blocks_per_sm<V, STAGE>(blocks_per_sm)) * ouro::host::sm_count();
+  const unsigned long long warps = 8ull * grid, requests = n_tasks << TASK_REQ_LOG;
+  unsigned round_log = 0;
+  for (unsigned t = ouro::host::round_task(requests, warps); t > 1; t >>= 1) ++round_log;
+  /* single rounds for the last two tasks' worth per warp */
+  const unsigned long long rounds = requests >> round_log, tail = (2 * warps) << (TASK_REQ_LOG - round_log);
+  k_batches_persistent<V, STAGE><<<grid, 256, 0, s>>>(H->d, d_sizes, d_offs, d_task_offs, n_batches, seed, mode, d_out,
+                                                      d_work, rounds, rounds > tail ? rounds - tail : 0, round_log);
+  OURO_LAUNCHED();
+  return OURO_OK;
+}
+
 template <int V>
 ouro_status batches_persistent(ouro_heap *H, const uint32_t *d_sizes, const unsigned long long *d_offs,
                                const unsigned long long *d_task_offs, uint32_t n_batches, uint64_t n_tasks,
                                uint32_t seed, int mode, ouro_check *d_out, unsigned long long *d_work,
                                int blocks_per_sm, cudaStream_t s) {
-  if (H->d.staging) {
-    const int per_sm = std::max(1, persistent_blocks_per_sm<V, true>(blocks_per_sm));
-    k_batches_persistent<V, true><<<per_sm * ouro::host::sm_count(), 256, 0, s>>>(
-        H->d, d_sizes, d_offs, d_task_offs, n_batches, seed, mode, d_out, d_work, n_tasks);
-  } else {
-    const int per_sm = std::max(1, persistent_blocks_per_sm<V, false>(blocks_per_sm));
-    k_batches_persistent<V, false><<<per_sm * ouro::host::sm_count(), 256, 0, s>>>(
-        H->d, d_sizes, d_offs, d_task_offs, n_batches, seed, mode, d_out, d_work, n_tasks);
-  }
-  OURO_LAUNCHED();
-  return OURO_OK;
+  return H->d.staging ? batches_form<V, true>(H, d_sizes, d_offs, d_task_offs, n_batches, n_tasks, seed, mode, d_out,
+                                              d_work, blocks_per_sm, s)
+                      : batches_form<V, false>(H, d_sizes, d_offs, d_task_offs, n_batches, n_tasks, seed, mode, d_out,
+                                               d_work, blocks_per_sm, s);
 }
 
 /* blocks of 256 per SM the unstaged persistent kernel keeps resident */
