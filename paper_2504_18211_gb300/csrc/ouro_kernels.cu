@@ -40,9 +40,11 @@ __global__ void k_batch_free(ouro_heap_dev h, void *const *ptrs, size_t n) {
  *
  * Each thread carries R requests (r * 256 + thread of the block's span, so
  * loads coalesce).  On plain-array queues a thread first tries all R of its
- * positions at once: R relaxed slot loads (malloc) or R relaxed slot CASes
- * (free) in flight together, behind one acquire / release fence, instead of
- * R chains of dependent round trips.  A position whose slot is not ready
+ * positions at once, pages and runs: R relaxed slot loads (malloc) or R
+ * relaxed slot CASes (free) in flight together, behind one acquire / release
+ * fence, instead of R chains of dependent round trips.  (With 2 % runs among
+ * 2^20 requests every other warp went through the warp path for them: malloc
+ * 28.6 us, 24 so.)  A position whose slot is not ready
  * (not produced yet, or its previous lap not consumed yet) goes through the
  * warp path with the position already taken, which waits, carves and
  * answers as ouro_malloc / ouro_free do. */
@@ -100,15 +102,22 @@ __global__ void __launch_bounds__(256, 4) k_batch_malloc_blk(ouro_heap_dev h, co
       unsigned long long v[R];
 #pragma unroll
       for (int r = 0; r < R; ++r)
-        v[r] = pend[r] && cls[r] < (int)h.n_classes ? ld_rlx(s_ring[cls[r]] + (pos[r] & s_rmask[cls[r]])) : 0ull;
+        v[r] = pend[r] ? ld_rlx(s_ring[cls[r]] + (pos[r] & s_rmask[cls[r]])) : 0ull;
       fence_acq_rel();
 #pragma unroll
       for (int r = 0; r < R; ++r) {
-        if (!pend[r] || cls[r] >= (int)h.n_classes) continue;
+        if (!pend[r]) continue;
         const int d = slot_d(v[r], pos[r]);
         if (d == 1 || d == 2) {   /* an item, or the heap's null answer: take it, retire the slot */
           st_rlx(s_ring[cls[r]] + (pos[r] & s_rmask[cls[r]]), slot(pos[r] + s_rmask[cls[r]] + 1, 0));
-          if (d == 1) res[r] = h.base + ((size_t)lo32(v[r]) << (4 + cls[r]));
+          if (d == 1) {
+            unsigned sh = 4u + cls[r];
+            if (cls[r] >= (int)h.n_classes) {   /* a run: the item is its first chunk, live again */
+              h.chunk_cls[lo32(v[r])] = (unsigned char)cls[r];
+              sh = h.log2_chunk;
+            }
+            res[r] = h.base + ((size_t)lo32(v[r]) << sh);
+          }
           pend[r] = false;
         }
       }
