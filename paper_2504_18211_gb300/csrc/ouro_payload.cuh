@@ -49,12 +49,20 @@ __device__ __forceinline__ int free_locate(const ouro_heap_dev &h, void *p, unsi
 }
 
 /* FENCE = false: only for kernels that free blocks written before they began
- * and allocate nothing (the batch free kernel) */
+ * and allocate nothing (the batch free kernel).  known_cls >= 0: the caller
+ * allocated p itself with that class; a page's chunk-table lookup (one L2
+ * round trip) is then left out, as in stage_free. */
 template <int V, bool FENCE = true>
-__device__ __forceinline__ void free_v(const ouro_heap_dev &h, void *p) {
+__device__ __forceinline__ void free_v(const ouro_heap_dev &h, void *p, int known_cls = -1) {
   const unsigned mask = __activemask();
   unsigned item = 0;
-  const int cls = free_locate<V>(h, p, item);
+  int cls;
+  if (p && known_cls >= 0 && known_cls < (int)h.n_classes && !(ouro_page_queues(V) && h.checked)) {
+    cls = known_cls;
+    item = (unsigned)(((const unsigned char *)p - h.base) >> (4 + cls));
+  } else {
+    cls = free_locate<V>(h, p, item);
+  }
   if constexpr (!ouro_page_queues(V)) {
     chunk_or_run_free<V, FENCE>(h, cls, item, p, mask);
   } else {

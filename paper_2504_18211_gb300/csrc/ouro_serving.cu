@@ -53,7 +53,7 @@ struct serve_args {
   /* results */
   unsigned long long *sess_out;  /* per session: xor, sum, mismatches, admit step, done step (u64 each) */
   unsigned long long *step_ns;   /* per step: %globaltimer after admission, growth and completion (3 words) */
-  unsigned long long *ctl;       /* [0] barrier count, [1] barrier generation, [2] next arrival,
+  unsigned long long *ctl;       /* [0] barrier arrivals, [1] reserved, [2] next arrival,
                                     [3] committed blocks, [4] error, [5] mallocs, [6] frees, [7] failed,
                                     [8] free-slot stack top, [9 + step % 2] sessions finished this step */
   uint32_t *free_stack;          /* free slot ids (stack of n_slots) */
@@ -71,30 +71,32 @@ __device__ __forceinline__ unsigned long long globaltimer() {
   return t;
 }
 
-/* grid barrier for a cooperative launch; a wait that runs out sets ctl[4] */
-__device__ bool grid_barrier(unsigned long long *ctl, unsigned nblocks, unsigned limit) {
+/* Grid barrier for a cooperative launch: ctl[0] counts arrivals and is never
+ * reset, the e-th barrier waits until it reaches e * nblocks, so an arrival is
+ * one fence and one atomic, and the wait polls that same word.  A wait that
+ * runs out sets ctl[4] and BARRIER_FAILED in the count, which ends every other
+ * block's wait. */
+constexpr unsigned long long BARRIER_FAILED = 1ull << 62;
+
+__device__ bool grid_barrier(unsigned long long *ctl, unsigned nblocks, unsigned limit, unsigned &epoch) {
   __shared__ int ok;
   __syncthreads();
+  ++epoch;
   if (threadIdx.x == 0) {
-    ok = 1;
-    const unsigned long long gen = ld_acq(&ctl[1]);
+    const unsigned long long target = (unsigned long long)nblocks * epoch;
     __threadfence();
-    if (atomicAdd(&ctl[0], 1ull) == nblocks - 1) {
-      st_rlx(&ctl[0], 0ull);
-      __threadfence();
-      atomicAdd(&ctl[1], 1ull);
-    } else {
-      unsigned it = 0;
-      while (ld_acq(&ctl[1]) == gen) {
-        if (++it > limit) {
-          atomicExch(&ctl[4], 1ull);
-          ok = 0;
-          break;
-        }
-        __nanosleep(32);
+    unsigned long long seen = atomicAdd(&ctl[0], 1ull) + 1;
+    if (seen >= target) __threadfence();
+    for (unsigned it = 0; seen < target; seen = ld_acq(&ctl[0])) {
+      if (++it > limit) {
+        atomicExch(&ctl[4], 1ull);
+        atomicAdd(&ctl[0], BARRIER_FAILED);
+        seen = BARRIER_FAILED;
+        break;
       }
+      __nanosleep(32);
     }
-    if (ld_acq(&ctl[4])) ok = 0;
+    ok = seen < BARRIER_FAILED;
   }
   __syncthreads();
   return ok != 0;
@@ -158,12 +160,24 @@ __device__ void serve_admit(const serve_args &A, uint32_t step) {
  * in flight per lane.  One warp per session had walked the allocator's chain
  * and 16 KiB alone, sessions one after another.  What is left is a chain of
  * L2 round trips, not bandwidth: 400 steps of about 1700 blocks of 16 KiB took
- * 12.3 ms with five barriers and phases a step, 8.0 ms so (28 MB a step would
- * take 4.2 us of its 20 at the copy rate). */
+ * 12.3 ms with five barriers and phases a step, 8.0 ms so, 6.9 ms with the
+ * sessions kept and grid_barrier on one word (28 MB a step would take 4.2 us of its
+ * 17 at the copy rate). */
 constexpr uint32_t SERVE_PIECE = 256;
 
+/* a lane's session between two steps of one launch */
+struct serve_lane {
+  unsigned long long x, sum, mism;
+  int sess;                /* -1: none */
+  uint32_t k, total;
+};
+
+/* keep (shared memory, one entry per lane of the first warp; null in the
+ * per-launch form): the block's sessions stay there from step to step, for
+ * grids that hold every slot at once, instead of being read back from memory
+ * (two dependent L2 round trips a step). */
 template <int V>
-__device__ void serve_grow(const serve_args &A, uint32_t step) {
+__device__ void serve_grow(const serve_args &A, uint32_t step, serve_lane *keep) {
   __shared__ unsigned char *s_bp[32];
   __shared__ uint32_t s_key[32];
   __shared__ unsigned long long s_sum[32];
@@ -180,11 +194,21 @@ __device__ void serve_grow(const serve_args &A, uint32_t step) {
     unsigned at = 0;
     if (warp == 0) {
       slot = first + (unsigned long long)lane * gridDim.x;
-      if (slot < A.n_slots) sess = __ldcg(&A.slot_session[slot]);
-      fresh = sess < -1;
-      if (fresh) sess = -2 - sess;
-      if (sess >= 0) {
-        total = A.blocks[sess];
+      if (keep && keep[lane].sess >= 0) {
+        const serve_lane l = keep[lane];
+        sess = l.sess;
+        k = l.k;
+        total = l.total;
+        x = l.x;
+        sum = l.sum;
+        mism = l.mism;
+      } else if (slot < A.n_slots) {
+        sess = __ldcg(&A.slot_session[slot]);
+        fresh = sess < -1;
+        if (fresh) sess = -2 - sess;
+        if (sess >= 0) total = A.blocks[sess];
+      }
+      if (!keep && sess >= 0) {
         if (!fresh) {
           k = A.slot_k[slot];
           x = A.slot_acc[3 * slot];
@@ -253,13 +277,21 @@ __device__ void serve_grow(const serve_args &A, uint32_t step) {
         sum += s_sum[at];
         mism += s_mism[at];
       }
-      A.slot_k[slot] = k;
-      if (k < total) {
+      if (!keep || k >= total) A.slot_k[slot] = k;
+      if (keep) {
+        keep[lane].sess = k < total ? sess : -1;
+        keep[lane].k = k;
+        keep[lane].total = total;
+        keep[lane].x = x;
+        keep[lane].sum = sum;
+        keep[lane].mism = mism;
+      }
+      if (k < total && !keep) {
         if (fresh) A.slot_session[slot] = sess;
         A.slot_acc[3 * slot] = x;
         A.slot_acc[3 * slot + 1] = sum;
         A.slot_acc[3 * slot + 2] = mism;
-      } else {   /* complete: report, release the slot (reused from the next step on), list it for freeing */
+      } else if (k >= total) {   /* complete: report, release the slot (reused from the next step on), list it for freeing */
         A.sess_out[5ull * sess + 0] = x;
         A.sess_out[5ull * sess + 1] = sum;
         A.sess_out[5ull * sess + 2] = mism;
@@ -289,6 +321,7 @@ __device__ void serve_free(const serve_args &A, uint32_t step) {
   const unsigned lane = laneid();
   const unsigned long long nwarps = (gridDim.x * blockDim.x) >> 5;
   const ouro_heap_dev &h = A.h;
+  const int cls = size_class(h, A.block_bytes);   /* of every block in the tables */
   const unsigned long long nl = *(volatile unsigned long long *)&A.ctl[9 + (step & 1)];
   for (unsigned long long c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;; c += nwarps) {
     unsigned long long before = 0;
@@ -319,7 +352,7 @@ __device__ void serve_free(const serve_args &A, uint32_t step) {
     for (uint32_t b0 = b_lo; b0 < b_hi; b0 += 32) {
       const uint32_t b = b0 + lane;
       void *p = b < b_hi ? reinterpret_cast<void *>(__ldcg(&A.tables[(size_t)slot * A.max_blocks + b])) : nullptr;
-      if (b < b_hi) free_v<V>(h, p);
+      if (b < b_hi) free_v<V>(h, p, cls);
       __syncwarp();
     }
   }
@@ -330,19 +363,23 @@ __device__ void serve_free(const serve_args &A, uint32_t step) {
  * has grown and when its frees and the next admission are done. */
 template <int V>
 __global__ void __launch_bounds__(256, 2) k_serve(serve_args A) {
+  unsigned epoch = 0;
   serve_init(A);
-  if (!grid_barrier(A.ctl, gridDim.x, A.spin_limit)) return;
+  if (!grid_barrier(A.ctl, gridDim.x, A.spin_limit, epoch)) return;
   if (A.steps) serve_admit(A, 0);
-  if (!grid_barrier(A.ctl, gridDim.x, A.spin_limit)) return;
+  if (!grid_barrier(A.ctl, gridDim.x, A.spin_limit, epoch)) return;
   const bool stamps = blockIdx.x == 0 && threadIdx.x == 0;
+  __shared__ serve_lane lanes[32];
+  serve_lane *keep = A.n_slots <= 32ull * gridDim.x ? lanes : nullptr;
+  if (threadIdx.x < 32) lanes[threadIdx.x].sess = -1;
   for (uint32_t step = 0; step < A.steps; ++step) {
     if (stamps) A.step_ns[3 * step] = globaltimer();
-    serve_grow<V>(A, step);
-    if (!grid_barrier(A.ctl, gridDim.x, A.spin_limit)) return;
+    serve_grow<V>(A, step, keep);
+    if (!grid_barrier(A.ctl, gridDim.x, A.spin_limit, epoch)) return;
     if (stamps) A.step_ns[3 * step + 1] = globaltimer();
     if (step + 1 < A.steps) serve_admit(A, step + 1);
     serve_free<V>(A, step);
-    if (!grid_barrier(A.ctl, gridDim.x, A.spin_limit)) return;
+    if (!grid_barrier(A.ctl, gridDim.x, A.spin_limit, epoch)) return;
     if (stamps) A.step_ns[3 * step + 2] = globaltimer();
   }
 }
@@ -362,7 +399,7 @@ __global__ void __launch_bounds__(256, 2) k_serve_phase(serve_args A, uint32_t s
   }
   if (PH == PH_INIT) serve_init(A);
   if (PH == PH_ADMIT) serve_admit(A, step);
-  if (PH == PH_GROW) serve_grow<V>(A, step);
+  if (PH == PH_GROW) serve_grow<V>(A, step, nullptr);
   if (PH == PH_FREE) {
     if (step + 1 < A.steps) serve_admit(A, step + 1);
     serve_free<V>(A, step);
