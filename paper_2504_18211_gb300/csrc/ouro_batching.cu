@@ -120,7 +120,7 @@ ouro_status batches_form(ouro_heap *H, const uint32_t *d_sizes, const unsigned l
   const int grid = std::max(1, persistent_blocks_per_sm<V, STAGE>(blocks_per_sm)) * ouro::host::sm_count();
   const unsigned long long warps = 8ull * grid, requests = n_tasks << TASK_REQ_LOG;
   unsigned round_log = 0;
-  for (unsigned t = ouro::host::round_task(requests, warps); t > 1; t >>= 1) ++round_log;
+  for (unsigned t = ouro::host::round_task(requests, warps, ouro_page_queues(V)); t > 1; t >>= 1) ++round_log;
   /* single rounds for the last two tasks' worth per warp */
   const unsigned long long rounds = requests >> round_log, tail = (2 * warps) << (TASK_REQ_LOG - round_log);
   k_batches_persistent<V, STAGE><<<grid, 256, 0, s>>>(H->d, d_sizes, d_offs, d_task_offs, n_batches, seed, mode, d_out,

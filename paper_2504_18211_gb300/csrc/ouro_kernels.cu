@@ -632,7 +632,7 @@ template <int V, bool STAGE>
 ouro_status round_fused_form(ouro_heap *H, const uint32_t *d_sizes, size_t n, uint32_t seed, int mode,
                              ouro_check *d_out, void **d_ptrs, void *work, cudaStream_t s) {
   const int block = 256, cap = occupancy_grid(k_round_fused<V, STAGE>, block);
-  const unsigned task = ouro::host::round_task(n, (size_t)cap * (block / 32));
+  const unsigned task = ouro::host::round_task(n, (size_t)cap * (block / 32), ouro_page_queues(V));
   k_round_fused<V, STAGE><<<grid_for((n + task - 1) / task * 32, block, cap), block, 0, s>>>(
       H->d, d_sizes, n, seed, mode, task, d_out, d_ptrs, static_cast<work_slot *>(work));
   OURO_LAUNCHED();
