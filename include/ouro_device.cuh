@@ -2053,62 +2053,78 @@ __device__ void *chunk_malloc(const ouro_heap_dev &h, int cls, unsigned vmask) {
   return ret;
 }
 
-/* The release half of a chunk-queue free: every lane of mask calls; lanes
- * with cls < 0 only take part.  Sets the page's bit and counts it back on
- * its chunk; true for the lane whose count increment lifted the chunk from
- * <= 0 to >= 1 (that lane queues chunk x).  cls turns to -1 on a double
- * free (recorded).  FENCE = false: the caller's blocks were written before
- * the kernel began and no malloc runs in the same kernel (the batch free
- * kernels), so no release is needed */
-template <bool FENCE = true>
-__device__ bool chunk_release(const ouro_heap_dev &h, int &cls, const void *p, unsigned mask, unsigned &x) {
+/* The release half of R chunk-queue frees per lane: every lane of mask calls;
+ * entries with cls < 0 only take part.  Sets each page's bit and counts it
+ * back on its chunk; lift[r]: this lane's count increment lifted chunk x[r]
+ * from <= 0 to >= 1 (that lane queues the chunk).  cls[r] turns to -1 on a
+ * double free (recorded).  All R bit atomics of a lane are in flight together,
+ * then all R count atomics, so R frees take two L2 round trips and not 2 R.
+ * FENCE = false: the caller's blocks were written before the kernel began and
+ * no malloc runs in the same kernel (the batch free kernels), so no release is
+ * needed */
+template <int R, bool FENCE, typename P>
+__device__ __forceinline__ void chunk_release_n(const ouro_heap_dev &h, int (&cls)[R], P (&p)[R], unsigned mask,
+                                                unsigned (&x)[R], bool (&lift)[R]) {
   const unsigned lane = laneid();
-  unsigned pg = 0;
-  x = 0;
-  if (cls >= 0) {
-    const unsigned long long off = (unsigned long long)((const unsigned char *)p - h.base);
-    x = (unsigned)(off >> h.log2_chunk);
-    pg = (unsigned)((off & (h.chunk_bytes - 1)) >> (4 + cls));
-  }
+  unsigned bit[R], wg[R], old[R];
   /* 1. set the page bits, one atomicOr per (chunk, word) group; the fence
    * releases the block's data (and, after a warp barrier, the data other
    * lanes wrote into it) before the page can be claimed again */
   if (FENCE) fence_acq_rel();
-  const unsigned long long wkey = cls >= 0 ? (((unsigned long long)x << 32) | (pg >> 5)) : ~0ull;
-  const unsigned wg = warp_group(h, mask, wkey);
-  const unsigned bit = cls >= 0 ? 1u << (pg & 31) : 0u;
-  const unsigned bits = __reduce_or_sync(wg, bit);
-  unsigned old = 0;
-  if (cls >= 0 && lane == (unsigned)(__ffs(wg) - 1))
-    old = atomicOr(&h.bits[(size_t)x * h.words_per_chunk + (pg >> 5)], bits);
-  old = __shfl_sync(mask, old, __ffs(wg) - 1);
-  if (cls >= 0 && (old & bit)) {
-    set_error(h, OURO_ERR_DOUBLE_FREE, OURO_SITE_CHUNK_DOUBLE);
-    cls = -1;
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    unsigned pg = 0;
+    x[r] = 0;
+    if (cls[r] >= 0) {
+      const unsigned long long off = (unsigned long long)((const unsigned char *)p[r] - h.base);
+      x[r] = (unsigned)(off >> h.log2_chunk);
+      pg = (unsigned)((off & (h.chunk_bytes - 1)) >> (4 + cls[r]));
+    }
+    wg[r] = warp_group(h, mask, cls[r] >= 0 ? (((unsigned long long)x[r] << 32) | (pg >> 5)) : ~0ull);
+    bit[r] = cls[r] >= 0 ? 1u << (pg & 31) : 0u;
+    const unsigned bits = __reduce_or_sync(wg[r], bit[r]);
+    old[r] = 0;
+    if (cls[r] >= 0 && lane == (unsigned)(__ffs(wg[r]) - 1))
+      old[r] = atomicOr(&h.bits[(size_t)x[r] * h.words_per_chunk + (pg >> 5)], bits);
   }
-  /* 2. count the pages back per chunk; lifting the count from <= 0 queues it */
-  const unsigned cg = warp_group(h, mask, cls >= 0 ? x : OURO_NIL) & __ballot_sync(mask, cls >= 0);
-  bool lift = false;
-  if (cls >= 0 && lane == (unsigned)(__ffs(cg) - 1)) {
-    /* the count goes up after the bits are set (a reserving malloc that
-     * sees the count finds the bits, or waits for them in its claim) */
-    const int k = __popc(cg);
-    if (FENCE) fence_acq_rel();
-    const int b = atomicAdd(&h.chunk_free[x], k);
-    lift = b <= 0 && b + k >= 1;
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    old[r] = __shfl_sync(mask, old[r], __ffs(wg[r]) - 1);
+    if (cls[r] >= 0 && (old[r] & bit[r])) {
+      set_error(h, OURO_ERR_DOUBLE_FREE, OURO_SITE_CHUNK_DOUBLE);
+      cls[r] = -1;
+    }
   }
-  return lift;
+  /* 2. count the pages back per chunk, after the bits are set (a reserving
+   * malloc that sees the count finds the bits, or waits for them in its
+   * claim); lifting the count from <= 0 queues the chunk */
+  if (FENCE) fence_acq_rel();
+  int before[R];
+  unsigned k[R];
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const unsigned cg = warp_group(h, mask, cls[r] >= 0 ? x[r] : OURO_NIL) & __ballot_sync(mask, cls[r] >= 0);
+    const bool leads = cls[r] >= 0 && lane == (unsigned)(__ffs(cg) - 1);
+    k[r] = leads ? __popc(cg) : 0;
+    before[r] = leads ? atomicAdd(&h.chunk_free[x[r]], (int)k[r]) : 0;
+  }
+#pragma unroll
+  for (int r = 0; r < R; ++r) lift[r] = k[r] && before[r] <= 0 && before[r] + (int)k[r] >= 1;
 }
 
 /* free into a chunk queue: every lane of mask calls; lanes with cls < 0 only
- * take part (FENCE as for chunk_release) */
+ * take part (FENCE as for chunk_release_n) */
 template <int V, bool FENCE = true>
 __device__ void chunk_free_impl(const ouro_heap_dev &h, int cls, const void *p, unsigned mask) {
   constexpr int QF = ouro_qform(V);
   const unsigned lane = laneid();
-  unsigned x;
-  const bool lift = chunk_release<FENCE>(h, cls, p, mask, x);
-  push_group<QF>(h, cls, x, lift, mask);   /* the lifted chunks, one tail atomic per class */
+  int c1[1] = {cls};
+  const void *p1[1] = {p};
+  unsigned x[1];
+  bool lift[1];
+  chunk_release_n<1, FENCE>(h, c1, p1, mask, x, lift);
+  cls = c1[0];
+  push_group<QF>(h, cls, x[0], lift[0], mask);   /* the lifted chunks, one tail atomic per class */
   const unsigned sg = warp_group(h, mask, cls);
   if (cls >= 0 && lane == (unsigned)(__ffs(sg) - 1)) stat_add(h, cls, OURO_ST_FREE, __popc(sg));
 }
