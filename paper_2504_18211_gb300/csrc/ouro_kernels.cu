@@ -61,6 +61,7 @@ __device__ __forceinline__ void blk_reserve(const int (&cls)[R], unsigned long l
 template <int V, int R>
 __global__ void __launch_bounds__(256, 4) k_batch_malloc_blk(ouro_heap_dev h, const uint32_t *sizes, void **ptrs,
                                                              size_t n) {
+  ouro::chain_begin();
   constexpr bool RING = ouro_qform(V) == OURO_QF_RING;
   __shared__ unsigned s_cnt[OURO_MAX_CLASSES], s_ok[OURO_MAX_CLASSES];
   __shared__ unsigned long long s_pos[OURO_MAX_CLASSES];
@@ -152,6 +153,7 @@ __global__ void __launch_bounds__(256, 4) k_batch_malloc_blk(ouro_heap_dev h, co
 
 template <int V, int R>
 __global__ void __launch_bounds__(256) k_batch_free_blk(ouro_heap_dev h, void *const *ptrs, size_t n) {
+  ouro::chain_begin();
   constexpr bool RING = ouro_qform(V) == OURO_QF_RING;
   __shared__ unsigned s_cnt[OURO_MAX_CLASSES];
   __shared__ unsigned long long s_pos[OURO_MAX_CLASSES];
@@ -228,6 +230,7 @@ __global__ void __launch_bounds__(256) k_batch_free_blk(ouro_heap_dev h, void *c
  * this and the malloc below.) */
 template <int V, int R>
 __global__ void __launch_bounds__(256) k_batch_free_cblk(ouro_heap_dev h, void *const *ptrs, size_t n) {
+  ouro::chain_begin();
   constexpr bool RING = ouro_qform(V) == OURO_QF_RING;
   __shared__ unsigned s_cnt[OURO_MAX_CLASSES], s_free[OURO_MAX_CLASSES];
   __shared__ unsigned long long s_pos[OURO_MAX_CLASSES];
@@ -313,6 +316,7 @@ __global__ void __launch_bounds__(256) k_batch_free_cblk(ouro_heap_dev h, void *
 template <int V, int R>
 __global__ void __launch_bounds__(256, 2) k_batch_malloc_cblk(ouro_heap_dev h, const uint32_t *sizes, void **ptrs,
                                                            size_t n) {
+  ouro::chain_begin();
   constexpr bool RING = ouro_qform(V) == OURO_QF_RING;
   static_assert(256 * R < 2048, "task offsets and counts are 11-bit fields");
   constexpr unsigned MAX_TASKS = (256 * R) / 32 + OURO_MAX_CLASSES;   /* sum over classes of ceil(share / part) */
@@ -473,6 +477,7 @@ __device__ __forceinline__ void pattern_ids(void *const *ptrs, size_t n, payload
 template <int OP>
 __global__ void __launch_bounds__(256) k_pattern(void *const *ptrs, const uint32_t *sizes, size_t n, uint32_t seed,
                                                  int mode, size_t heads, unsigned task, ouro_check *out) {
+  ouro::chain_begin();
   __shared__ unsigned s_next;
   if (threadIdx.x == 0) s_next = 0;
   __syncthreads();
@@ -516,6 +521,7 @@ template <int V, bool STAGE>
 __global__ void __launch_bounds__(256, ouro_page_queues(V) ? OURO_FUSED_MIN_BLOCKS : 2) k_round_fused(ouro_heap_dev h, const uint32_t *sizes, size_t n,
                                                      uint32_t seed, int mode, unsigned task, ouro_check *out,
                                                      void **ptrs, work_slot *work) {
+  ouro::chain_begin();
   __shared__ ouro_block_ctx<8> ctx;
   if (STAGE) ouro_block_begin(ctx);
   payload_acc a;
@@ -627,13 +633,14 @@ ouro_status batch_malloc(ouro_heap *H, const uint32_t *d_sizes, void **d_ptrs, s
     if (!H->d.deopt) {
       if constexpr (ouro_qform(V) == OURO_QF_RING) {
         if (blk_wide(n)) {
-          k_batch_malloc_blk<V, BLK_WIDE><<<grid_for((n + BLK_WIDE - 1) / BLK_WIDE, block, 1 << 20), block, 0, s>>>(
-              H->d, d_sizes, d_ptrs, n);
+          ouro::host::launch_chained(k_batch_malloc_blk<V, BLK_WIDE>, grid_for((n + BLK_WIDE - 1) / BLK_WIDE, block, 1 << 20), block, s,
+                                       H->d, d_sizes, d_ptrs, n);
           OURO_LAUNCHED();
           return OURO_OK;
         }
       }
-      k_batch_malloc_blk<V, 1><<<grid_for(n, block, 1 << 20), block, 0, s>>>(H->d, d_sizes, d_ptrs, n);
+      ouro::host::launch_chained(k_batch_malloc_blk<V, 1>, grid_for(n, block, 1 << 20), block, s,
+                                       H->d, d_sizes, d_ptrs, n);
       OURO_LAUNCHED();
       return OURO_OK;
     }
@@ -641,10 +648,11 @@ ouro_status batch_malloc(ouro_heap *H, const uint32_t *d_sizes, void **d_ptrs, s
   if constexpr (!ouro_page_queues(V)) {
     if (!H->d.deopt) {
       if (blk_wide(n))
-        k_batch_malloc_cblk<V, BLK_WIDE><<<grid_for((n + BLK_WIDE - 1) / BLK_WIDE, block, 1 << 20), block, 0, s>>>(
-            H->d, d_sizes, d_ptrs, n);
+        ouro::host::launch_chained(k_batch_malloc_cblk<V, BLK_WIDE>, grid_for((n + BLK_WIDE - 1) / BLK_WIDE, block, 1 << 20), block, s,
+                                       H->d, d_sizes, d_ptrs, n);
       else
-        k_batch_malloc_cblk<V, 1><<<grid_for(n, block, 1 << 20), block, 0, s>>>(H->d, d_sizes, d_ptrs, n);
+        ouro::host::launch_chained(k_batch_malloc_cblk<V, 1>, grid_for(n, block, 1 << 20), block, s,
+                                       H->d, d_sizes, d_ptrs, n);
       OURO_LAUNCHED();
       return OURO_OK;
     }
@@ -661,19 +669,20 @@ ouro_status batch_free(ouro_heap *H, void *const *d_ptrs, size_t n, cudaStream_t
     if (!H->d.deopt) {
       if constexpr (ouro_qform(V) == OURO_QF_RING) {
         if (free_wide(n)) {
-          k_batch_free_blk<V, FREE_WIDE>
-              <<<grid_for((n + FREE_WIDE - 1) / FREE_WIDE, FREE_BLOCK, 1 << 20), FREE_BLOCK, 0, s>>>(H->d, d_ptrs, n);
+          ouro::host::launch_chained(k_batch_free_blk<V, FREE_WIDE>, grid_for((n + FREE_WIDE - 1) / FREE_WIDE, FREE_BLOCK, 1 << 20), FREE_BLOCK, s,
+                                       H->d, d_ptrs, n);
           OURO_LAUNCHED();
           return OURO_OK;
         }
         if (blk_wide(n)) {
-          k_batch_free_blk<V, BLK_WIDE><<<grid_for((n + BLK_WIDE - 1) / BLK_WIDE, block, 1 << 20), block, 0, s>>>(
-              H->d, d_ptrs, n);
+          ouro::host::launch_chained(k_batch_free_blk<V, BLK_WIDE>, grid_for((n + BLK_WIDE - 1) / BLK_WIDE, block, 1 << 20), block, s,
+                                       H->d, d_ptrs, n);
           OURO_LAUNCHED();
           return OURO_OK;
         }
       }
-      k_batch_free_blk<V, 1><<<grid_for(n, block, 1 << 20), block, 0, s>>>(H->d, d_ptrs, n);
+      ouro::host::launch_chained(k_batch_free_blk<V, 1>, grid_for(n, block, 1 << 20), block, s,
+                                       H->d, d_ptrs, n);
       OURO_LAUNCHED();
       return OURO_OK;
     }
@@ -681,10 +690,11 @@ ouro_status batch_free(ouro_heap *H, void *const *d_ptrs, size_t n, cudaStream_t
   if constexpr (!ouro_page_queues(V)) {
     if (!H->d.deopt) {
       if (blk_wide(n))
-        k_batch_free_cblk<V, BLK_WIDE><<<grid_for((n + BLK_WIDE - 1) / BLK_WIDE, block, 1 << 20), block, 0, s>>>(
-            H->d, d_ptrs, n);
+        ouro::host::launch_chained(k_batch_free_cblk<V, BLK_WIDE>, grid_for((n + BLK_WIDE - 1) / BLK_WIDE, block, 1 << 20), block, s,
+                                       H->d, d_ptrs, n);
       else
-        k_batch_free_cblk<V, 1><<<grid_for(n, block, 1 << 20), block, 0, s>>>(H->d, d_ptrs, n);
+        ouro::host::launch_chained(k_batch_free_cblk<V, 1>, grid_for(n, block, 1 << 20), block, s,
+                                       H->d, d_ptrs, n);
       OURO_LAUNCHED();
       return OURO_OK;
     }
@@ -699,8 +709,8 @@ ouro_status round_fused_form(ouro_heap *H, const uint32_t *d_sizes, size_t n, ui
                              ouro_check *d_out, void **d_ptrs, void *work, cudaStream_t s) {
   const int block = 256, cap = occupancy_grid(k_round_fused<V, STAGE>, block);
   const unsigned task = ouro::host::round_task(n, (size_t)cap * (block / 32), ouro_page_queues(V));
-  k_round_fused<V, STAGE><<<grid_for((n + task - 1) / task * 32, block, cap), block, 0, s>>>(
-      H->d, d_sizes, n, seed, mode, task, d_out, d_ptrs, static_cast<work_slot *>(work));
+  ouro::host::launch_chained(k_round_fused<V, STAGE>, grid_for((n + task - 1) / task * 32, block, cap), block, s,
+                             H->d, d_sizes, n, seed, mode, task, d_out, d_ptrs, static_cast<work_slot *>(work));
   OURO_LAUNCHED();
   return OURO_OK;
 }
@@ -748,7 +758,7 @@ extern "C" ouro_status ouro_pattern_write(void *const *d_ptrs, const uint32_t *d
   if (!n) return OURO_OK;
   const int block = 256;
   const pattern_shape sh(n, mode, block, occupancy_grid(k_pattern<PAY_WRITE>, block));
-  k_pattern<PAY_WRITE><<<sh.grid, block, 0, S(stream)>>>(d_ptrs, d_sizes, n, seed, mode, sh.heads, sh.task, nullptr);
+  ouro::host::launch_chained(k_pattern<PAY_WRITE>, sh.grid, block, S(stream), d_ptrs, d_sizes, n, seed, mode, sh.heads, sh.task, nullptr);
   OURO_LAUNCHED();
   return OURO_OK;
 }
@@ -761,7 +771,7 @@ extern "C" ouro_status ouro_pattern_check(void *const *d_ptrs, const uint32_t *d
   if (!n) return OURO_OK;
   const int block = 256;
   const pattern_shape sh(n, mode, block, occupancy_grid(k_pattern<PAY_CHECK>, block));
-  k_pattern<PAY_CHECK><<<sh.grid, block, 0, S(stream)>>>(d_ptrs, d_sizes, n, seed, mode, sh.heads, sh.task, d_out);
+  ouro::host::launch_chained(k_pattern<PAY_CHECK>, sh.grid, block, S(stream), d_ptrs, d_sizes, n, seed, mode, sh.heads, sh.task, d_out);
   OURO_LAUNCHED();
   return OURO_OK;
 }
