@@ -168,7 +168,7 @@ __device__ void warp_append(const ouro_heap_dev &h, vertex *vx, const unsigned *
       }
       progress |= grow;
       __syncwarp();
-      free_v<V>(h, reinterpret_cast<void *>(old));
+      free_v<V>(h, reinterpret_cast<void *>(old), old ? size_class(h, 4ull * cap) : -1);
       __syncwarp();
     }
 
@@ -339,7 +339,10 @@ k_graph_insert(ouro_heap_dev h, vertex *vt, const unsigned *src, const unsigned 
  * vertex; the block's vertices with segments follow one by one, all threads
  * copying a segment while its link is read.  The chain of links bounds it: 86
  * of them for a list of 175,000 entries, which one warp alone copied in 1.3
- * ms (2^22 entries of 2^18 vertices: 1380 us so, 270 now). */
+ * ms (2^22 entries of 2^18 vertices: 1380 us so, 270 with the block, and less
+ * with its loads in flight past the ragged end of a segment, whose remainder
+ * loop had cost two of its threads seven round trips a segment; that and the
+ * free below took init, insert, gather, free and a sort from 1773 to 1593). */
 __global__ void __launch_bounds__(256) k_graph_gather(const vertex *vt, unsigned nv, const unsigned long long *off,
                                                       unsigned *out, unsigned chunk_bytes) {
   constexpr unsigned WARPS = 8;
@@ -372,8 +375,15 @@ __global__ void __launch_bounds__(256) k_graph_gather(const vertex *vt, unsigned
       for (unsigned k = 0; sg && k < (1u << 26); ++k) {
         const unsigned long long next = *reinterpret_cast<const unsigned long long *>(sg);
         const unsigned *e = reinterpret_cast<const unsigned *>(sg + 8);
-#pragma unroll 8
-        for (unsigned i = threadIdx.x; i < take; i += 256) out[o + i] = e[i];
+        for (unsigned i0 = threadIdx.x; i0 < take; i0 += 8 * 256) {   /* eight loads in flight, the ragged end too */
+          unsigned d[8];
+#pragma unroll
+          for (unsigned j = 0; j < 8; ++j)
+            if (i0 + 256 * j < take) d[j] = e[i0 + 256 * j];
+#pragma unroll
+          for (unsigned j = 0; j < 8; ++j)
+            if (i0 + 256 * j < take) out[o + i0 + 256 * j] = d[j];
+        }
         o += take;
         sg = next;
         take = seg_cap;
@@ -383,17 +393,32 @@ __global__ void __launch_bounds__(256) k_graph_gather(const vertex *vt, unsigned
   }
 }
 
+/* Frees every list.  A lane per vertex; the classes are known from the record,
+ * so no free reads the chunk table, and a segment's link is read before the
+ * frees of the segment before it wait for their queue slots. */
 template <int V>
 __global__ void k_graph_free(ouro_heap_dev h, vertex *vt, unsigned nv) {
-  for (unsigned v = blockIdx.x * blockDim.x + threadIdx.x; v < nv; v += gridDim.x * blockDim.x) {
-    free_v<V>(h, reinterpret_cast<void *>(vt[v].ptr));
-    unsigned long long seg = vt[v].ovf;
-    for (unsigned guard = 0; seg && guard < (1u << 26); ++guard) {
-      const unsigned long long nx = *reinterpret_cast<const unsigned long long *>(seg);
-      free_v<V>(h, reinterpret_cast<void *>(seg));
-      seg = nx;
+  const unsigned threads = gridDim.x * blockDim.x;
+  for (unsigned v0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31u); v0 < nv; v0 += threads) {
+    const unsigned v = v0 + (threadIdx.x & 31);
+    unsigned long long ptr = 0, seg = 0, end = 0;
+    if (v < nv) {
+      ptr = vt[v].ptr;
+      seg = vt[v].ovf;
+      end = vt[v].end;
     }
-    vt[v].ptr = vt[v].ovf = 0;
+    unsigned long long next = seg ? *reinterpret_cast<const unsigned long long *>(seg) : 0;
+    __syncwarp();
+    free_v<V>(h, reinterpret_cast<void *>(ptr), size_class(h, seg ? h.chunk_bytes : 4ull * hi32(end)));
+    for (unsigned guard = 0; __any_sync(0xffffffffu, seg != 0) && guard < (1u << 26); ++guard) {
+      const unsigned long long after = next ? *reinterpret_cast<const unsigned long long *>(next) : 0;
+      __syncwarp();
+      free_v<V>(h, reinterpret_cast<void *>(seg), (int)h.n_classes - 1);
+      __syncwarp();
+      seg = next;
+      next = after;
+    }
+    if (v < nv) vt[v].ptr = vt[v].ovf = 0;
   }
 }
 
