@@ -964,11 +964,11 @@ def extras(P, torch, np, heap, sizes, sizes_np, args, n, st, clk):
         return n / (t_same + t_dist), g
 
     # the batch kernels on page queues aggregate per block: 256 threads, four
-    # requests each on plain arrays once a batch fills every SM that way (as
-    # the library does); chunk queues aggregate per warp
+    # requests each once a batch fills every SM that way (as the library
+    # does); chunk queues aggregate per warp
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     if args.variant.startswith("page_"):
-        span = 256 * (4 if args.variant == "page_array" and n >= 4 * 256 * sms else 1)
+        span = 256 * (4 if n >= 4 * 256 * sms else 1)
     else:
         span = 32
     roof_pairs, g_blk = roof_pairs_for(span)

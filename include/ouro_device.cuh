@@ -173,6 +173,11 @@ __device__ __forceinline__ unsigned long long cas_rlx(unsigned long long *p, uns
                : "=l"(o) : "l"(p), "l"(c), "l"(v) : "memory");
   return o;
 }
+__device__ __forceinline__ unsigned long long exch_rlx(unsigned long long *p, unsigned long long v) {
+  unsigned long long o;
+  asm volatile("atom.relaxed.gpu.global.exch.b64 %0, [%1], %2;" : "=l"(o) : "l"(p), "l"(v) : "memory");
+  return o;
+}
 /* with a relaxed load before it, an acquire; with a relaxed write after it, a release */
 __device__ __forceinline__ void fence_acq_rel() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
 __device__ __forceinline__ unsigned long long cas_ar(unsigned long long *p, unsigned long long c,
@@ -607,14 +612,24 @@ static __device__ __noinline__ void vl_back_chase_warp(const ouro_heap_dev &h, o
   if (lane == 0) atomicMax(&q->back.v, pack(bi + run, xl));   /* indices only grow */
 }
 
+/* Every lane of the warp calls: the cells of segment idx in chunk x read empty
+ * for their own positions. */
+__device__ inline void seg_clear_warp(const ouro_heap_dev &h, unsigned x, unsigned idx) {
+  unsigned long long *cells = seg_cells(h, x);
+  const unsigned long long p0 = (unsigned long long)idx * h.seg_cap;
+  for (unsigned i = 2 * laneid(); i < h.seg_cap; i += 64)
+    *reinterpret_cast<ulonglong2 *>(cells + i) = make_ulonglong2(slot(p0 + i, 0), slot(p0 + i + 1, 0));
+}
+
 /* vl_append_run for a whole warp: the run's chunks are held as x[p] by lane
  * j % 32 for run offset j = 32 p + lane (j < k).  Lane 0 claims the back
  * segment's empty link; every lane sets its own segments up; lane 0
  * publishes the chain with one store; every lane then writes its segments'
  * lookaside hints.  A back hint that trails the list is moved up to 128
  * segments at a time; what finds no room goes to the spare stack as one
- * chain (one push). */
-template <int W>
+ * chain (one push).  FRESH: the chunks come from the heap, so their cells are
+ * initialised, by the whole warp, segment by segment. */
+template <int W, bool FRESH = false>
 static __device__ __noinline__ void vl_append_run_warp(const ouro_heap_dev &h, int c,
                                                        const unsigned (&x)[W], unsigned k,
                                                        unsigned long long &bk) {
@@ -674,11 +689,24 @@ static __device__ __noinline__ void vl_append_run_warp(const ouro_heap_dev &h, i
     b = __shfl_sync(0xffffffffu, b, 0);
     m = __shfl_sync(0xffffffffu, m, 0);
     const unsigned bi = hi32(b);
+    if (FRESH) {
+      for (unsigned j = placed; j < placed + m; ++j) {
+        const unsigned xj = vl_pick(x, j), idx = bi + 1 + (j - placed);
+        const unsigned nj = j + 1 < placed + m ? vl_pick(x, j + 1) : OURO_NIL;
+        seg_clear_warp(h, xj, idx);
+        if (lane == 0) {
+          seg_of(h, xj)->done = 0;
+          seg_of(h, xj)->link = pack(idx, nj);
+          OURO_TRACE_EVENT(OURO_TR_SEGMENT, c, idx, xj);
+        }
+      }
+    } else {
 #pragma unroll
-    for (int p = 0; p < W; ++p) {
-      const unsigned j = 32u * p + lane;
-      if (j >= placed && j < placed + m)
-        seg_setup(h, x[p], bi + 1 + (j - placed), false, j + 1 < placed + m ? nx[p] : OURO_NIL);
+      for (int p = 0; p < W; ++p) {
+        const unsigned j = 32u * p + lane;
+        if (j >= placed && j < placed + m)
+          seg_setup(h, x[p], bi + 1 + (j - placed), false, j + 1 < placed + m ? nx[p] : OURO_NIL);
+      }
     }
     __threadfence();
     const unsigned first = vl_pick(x, placed), last = vl_pick(x, placed + m - 1);
@@ -698,6 +726,13 @@ static __device__ __noinline__ void vl_append_run_warp(const ouro_heap_dev &h, i
     placed += m;
   }
   if (placed < k) {   /* the rest onto the spare stack, as one chain */
+    if (FRESH)        /* as segments of index 0: behind every position that they will serve */
+      for (unsigned j = placed; j < k; ++j) {
+        const unsigned xj = vl_pick(x, j);
+        seg_clear_warp(h, xj, 0);
+        if (lane == 0) seg_of(h, xj)->link = pack(0, OURO_NIL);
+      }
+    if (FRESH) __syncwarp();
 #pragma unroll
     for (int p = 0; p < W; ++p) {
       const unsigned j = 32u * p + lane;
@@ -1115,6 +1150,65 @@ static __device__ __noinline__ unsigned long long *vl_slot_walk(const ouro_heap_
   return nullptr;
 }
 
+/* Segments up to position `last` for a carve of list c, by the warp of the
+ * carve-lock holder (every lane calls): two or more that are missing are taken
+ * from the heap at once, set up by all lanes and linked behind the back as one
+ * chain, instead of by one lane in turn, a walk, a chunk and a thousand cells
+ * each.  With it and the tail rule of page_malloc the first burst on a cold
+ * list (3 * 2^18 requests, 25.4 ms) takes no longer in the block kernels'
+ * four-request form than it did with one request per thread; without the two
+ * 27.9.  Leaves the rest (a single segment, the first one, spares) to
+ * vl_slot. */
+static __device__ __noinline__ void vl_prepare_warp(const ouro_heap_dev &h, int c, unsigned long long last) {
+  ouro_qhdr *q = qh(h, c);
+  const unsigned lane = laneid();
+  unsigned ns = h.backoff_min_ns;
+  for (int tries = 0; tries < 64; ++tries) {
+    unsigned long long b = 0, link = 0;
+    unsigned need = 0;
+    int act = 0;   /* 0: nothing to do here, 1: append, 2: look again, 3: chase the back */
+    if (lane == 0) {
+      b = ld_acq(&q->back.v);
+      if (lo32(b) < OURO_BUSY && lo32(ld_rlx(&q->spare.v)) == OURO_NIL) {
+        const unsigned s = (unsigned)(last / h.seg_cap);
+        link = ld_acq(&seg_of(h, lo32(b))->link);
+        if (hi32(link) != hi32(b)) {
+          act = 2;
+        } else if ((int)(s - hi32(b)) >= 2) {
+          act = lo32(link) < OURO_BUSY ? 3 : lo32(link) == OURO_BUSY ? 2 : 1;
+          need = min(s - hi32(b), 32u);
+        }
+      }
+    }
+    act = __shfl_sync(0xffffffffu, act, 0);
+    if (act == 0) return;
+    if (act == 3) {
+      vl_back_chase_warp<1>(h, q, __shfl_sync(0xffffffffu, b, 0), lo32(__shfl_sync(0xffffffffu, link, 0)));
+      continue;
+    }
+    if (act == 2) {
+      backoff_wait(h, ns);
+      ns = min(ns * 2, h.backoff_max_ns);
+      continue;
+    }
+    chunk_range r{0, 0, 0, 0};
+    if (lane == 0) {
+      r = take_chunks(h, need);
+      stat_add(h, c, OURO_ST_SEG, r.k1 + r.k2);
+    }
+    r.p0 = __shfl_sync(0xffffffffu, r.p0, 0);
+    r.b0 = __shfl_sync(0xffffffffu, r.b0, 0);
+    r.k1 = __shfl_sync(0xffffffffu, r.k1, 0);
+    r.k2 = __shfl_sync(0xffffffffu, r.k2, 0);
+    const unsigned k = r.k1 + r.k2;
+    if (!k) return;   /* vl_slot records it */
+    unsigned x[1] = {lane < k ? range_chunk(h, r, lane) : OURO_NIL};
+    if (lane < k) h.chunk_cls[x[0]] = OURO_CLS_SEG;
+    unsigned long long bk = 0;
+    vl_append_run_warp<1, true>(h, c, x, k, bk);
+  }
+}
+
 /* slot of position pos for storage form QF (template-resolved) */
 template <int QF>
 __device__ __forceinline__ unsigned long long *slot_at(const ouro_heap_dev &h, int c,
@@ -1249,31 +1343,37 @@ __device__ void page_carve(const ouro_heap_dev &h, int c, unsigned vmask, int ow
   int exhausted = 0;
   unsigned long long t0 = 0;
   chunk_range r{0, 0, 0, 0};
+  unsigned long long t = 0, hd = 0, ask = 0, last = 0;   /* last: the last position whose segment this carve needs */
   if ((int)lane == owner) {
-    unsigned long long t = ld_acq(&q->tail.v), hd = ld_acq(&q->head.v);
+    t = ld_acq(&q->tail.v);
+    hd = ld_acq(&q->head.v);
     if (hd > t) {
       unsigned long long want = (hd - t + ppc - 1) >> ppc_log;
-      unsigned long long ask = min(want, (unsigned long long)h.max_carve);
+      ask = min(want, (unsigned long long)h.max_carve);
       ask = min(ask, max(1ull, (unsigned long long)(OURO_CARVE_SLOTS >> ppc_log)));
       if (V == OURO_PAGE_ARRAY) {
         unsigned long long limit = h.qcap[c] >> ppc_log, have = ld_rlx(&q->carved.v);
         ask = have >= limit ? 0 : min(ask, limit - have);
       }
-      if (VL) {
-        /* queue storage first: segments for every slot this carve (or its
-         * null answers) will write, before the data chunks are taken */
-        unsigned long long last = max(hd, t + (ask << ppc_log)) - 1;
-        seg_prepare<QF>(h, c, t, last);
-      }
-      if (ask) r = take_chunks(h, (unsigned)ask);
-      m = r.k1 + r.k2;
-      exhausted = m < ask || ask == 0;
-      if (m) {
-        t0 = atomicAdd(&q->tail.v, (unsigned long long)m << ppc_log);
-        atomicAdd(&q->carved.v, (unsigned long long)m);
-        stat_add(h, c, OURO_ST_CARVE, m);
-        OURO_TRACE_EVENT(OURO_TR_CARVE, c, m, t0);
-      }
+      last = max(hd, t + (ask << ppc_log)) - 1;
+    }
+  }
+  if (QF == OURO_QF_LIST && vmask == 0xffffffffu) {
+    const unsigned long long l = __shfl_sync(vmask, last, owner);
+    if (l) vl_prepare_warp(h, c, l);
+  }
+  if ((int)lane == owner && hd > t) {
+    /* queue storage first: segments for every slot this carve (or its null
+     * answers) will write, before the data chunks are taken */
+    if (VL) seg_prepare<QF>(h, c, t, last);
+    if (ask) r = take_chunks(h, (unsigned)ask);
+    m = r.k1 + r.k2;
+    exhausted = m < ask || ask == 0;
+    if (m) {
+      t0 = atomicAdd(&q->tail.v, (unsigned long long)m << ppc_log);
+      atomicAdd(&q->carved.v, (unsigned long long)m);
+      stat_add(h, c, OURO_ST_CARVE, m);
+      OURO_TRACE_EVENT(OURO_TR_CARVE, c, m, t0);
     }
   }
   unsigned long long dt = 0, dn = 0;
@@ -1459,7 +1559,8 @@ __device__ void *page_malloc(const ouro_heap_dev &h, int cls, unsigned vmask, un
   const unsigned grp = warp_group(h, vmask, cls);
   const unsigned leader = __ffs(grp) - 1;
   const unsigned rank = __popc(grp & lanemask_lt());
-  unsigned long long pos = 0;
+  unsigned long long pos = 0, tail0 = 0;
+  if (VL && req && lane == leader) tail0 = ld_rlx(&q->tail.v);   /* in flight beside the head atomic */
   if (RESERVED) pos = p_reserved;    /* the caller took this lane's head position (block aggregation) */
   else if (req && lane == leader) pos = atomicAdd(&q->head.v, (unsigned long long)__popc(grp));
   const unsigned long long p0 = __shfl_sync(vmask, pos, leader);   /* the group leader's position */
@@ -1469,10 +1570,14 @@ __device__ void *page_malloc(const ouro_heap_dev &h, int cls, unsigned vmask, un
   int st = req ? 0 : 3;   /* 0 waiting, 1 item, 2 null answer, 3 gave up (helpers: nothing asked) */
   unsigned long long *cell = nullptr;
   if (VL) {   /* the leader finds its segment; lanes in the same segment reuse it */
-    unsigned long long *c0 = (req && lane == leader) ? slot_at<QF>(h, cls, p0, false) : nullptr;
+    /* positions past the tail have no producer yet: their segment is not
+     * looked for (thousands of waiting warps that walked the list for it
+     * slowed the one that carves) */
+    tail0 = __shfl_sync(vmask, tail0, leader);
+    unsigned long long *c0 = (req && lane == leader && p0 < tail0) ? slot_at<QF>(h, cls, p0, false) : nullptr;
     c0 = reinterpret_cast<unsigned long long *>(
         __shfl_sync(vmask, reinterpret_cast<unsigned long long>(c0), leader));
-    if (req)
+    if (req && pos < tail0)
       cell = (c0 && pos / h.seg_cap == p0 / h.seg_cap) ? c0 + (long long)(pos - p0) : slot_at<QF>(h, cls, pos, false);
   } else if (req) {
     cell = ring_slot(h, cls, pos);
@@ -1485,10 +1590,15 @@ __device__ void *page_malloc(const ouro_heap_dev &h, int cls, unsigned vmask, un
     for (unsigned it = 0;; ++it) {
       bool debt = false, progressed = false;
       if (st == 0) {
-        if (VL && !cell) cell = slot_at<QF>(h, cls, pos, false);
-        if (cell) st = try_take<VL>(h, cls, cell, pos, &item);
+        if (VL && !cell) {
+          debt = pos >= ld_acq(&q->tail.v);
+          if (!debt) cell = slot_at<QF>(h, cls, pos, false);
+          if (cell) st = try_take<VL>(h, cls, cell, pos, &item);
+        } else {
+          if (cell) st = try_take<VL>(h, cls, cell, pos, &item);
+          if (!st) debt = pos >= ld_acq(&q->tail.v);
+        }
         if (st) progressed = true;
-        else debt = pos >= ld_acq(&q->tail.v);
       }
       const unsigned dmask = __ballot_sync(vmask, debt);
       if (dmask) {

@@ -11,6 +11,8 @@
  * 16-byte units that the 32 lanes write and read in turn, so stores and
  * loads are 16-byte vectors that coalesce within each block.
  */
+#include <type_traits>
+
 #include "ouro_internal.cuh"
 #include "ouro_payload.cuh"
 #include "ouro_shard.cuh"
@@ -58,11 +60,114 @@ __device__ __forceinline__ void blk_reserve(const int (&cls)[R], unsigned long l
     pos[r] = cls[r] >= 0 ? atomicAdd(&s_cnt[cls[r]], 1u) : 0u;
 }
 
+/* block of a taken item: a page id, or a run's first chunk, which is live again */
+__device__ __forceinline__ void *blk_block(const ouro_heap_dev &h, int cls, unsigned item) {
+  unsigned sh = 4u + cls;
+  if (cls >= (int)h.n_classes) {
+    h.chunk_cls[item] = (unsigned char)cls;
+    sh = h.log2_chunk;
+  }
+  return h.base + ((size_t)item << sh);
+}
+
+/* Segments under a block's share of each class (virtualized queues, several
+ * requests per thread): the share's positions are consecutive, so they lie in
+ * at most BLK_SEGS segments unless the chunks are small.  One thread per class
+ * and segment looks its segment up, all at once; every request then finds its
+ * slot by offset, and the block counts its position events on a segment with
+ * one atomic.  A share's further segments, and a segment that is not there
+ * yet, are left to the warp path.  (3 * 2^18 requests of 64 B on a list,
+ * malloc, write, check and free: 127 us with one request per thread and a
+ * lookup per warp, 118 so.) */
+constexpr unsigned BLK_SEGS = 4;
+struct blk_segs {
+  unsigned long long *cells[OURO_MAX_CLASSES][BLK_SEGS];   /* slot 0 of the segment; null: not known */
+  unsigned events[OURO_MAX_CLASSES][BLK_SEGS];
+  unsigned off0[OURO_MAX_CLASSES];                         /* offset of the share's first position */
+  unsigned long long end[OURO_MAX_CLASSES];                /* consumers: the class's tail; further segments may not exist */
+  unsigned retire;                                         /* classes with a segment to retire (lists) */
+};
+
+/* After the block's positions are taken; ends with a block barrier.  CREATE:
+ * producers, who make missing segments and look ahead as va_slot / vl_slot do. */
+template <int QF, bool CREATE>
+__device__ void blk_segs_find(const ouro_heap_dev &h, blk_segs &sg, const unsigned *cnt, const unsigned long long *pos) {
+  static_assert(OURO_MAX_CLASSES * BLK_SEGS <= 128, "a thread per class and segment of the smallest block");
+  if (threadIdx.x < OURO_MAX_CLASSES * BLK_SEGS) {
+    const unsigned c = threadIdx.x / BLK_SEGS, j = threadIdx.x % BLK_SEGS;
+    unsigned long long *cells = nullptr;
+    if (cnt[c]) {
+      const unsigned long long s0 = pos[c] / h.seg_cap, s = s0 + j;
+      const unsigned off0 = (unsigned)(pos[c] - s0 * h.seg_cap), end = off0 + cnt[c];   /* offsets from s0's slot 0 */
+      if (j == 0) sg.off0[c] = off0;
+      if (j * h.seg_cap < end && (CREATE || s * h.seg_cap < sg.end[c])) {
+        const unsigned lo = j ? 0 : off0, hi = min(end - j * h.seg_cap, h.seg_cap);   /* the share in segment s: [lo, hi) */
+        unsigned long long *cell = slot_at<QF>(h, (int)c, s * h.seg_cap + lo, CREATE);
+        if (cell) {
+          cells = cell - lo;
+          const unsigned w = h.seg_cap >> 3;
+          if (CREATE && lo < w && hi > w) {   /* the look-ahead of the positions just past 1/8 of the segment */
+            if (QF == OURO_QF_VARRAY) va_prefetch(h, (int)c, (unsigned)s + 1);
+            else vl_prefetch(h, (int)c, pack((unsigned)s, (unsigned)(((const unsigned char *)cell - h.base) >> h.log2_chunk)));
+          }
+        }
+      }
+    }
+    sg.cells[c][j] = cells;
+    sg.events[c][j] = 0;
+    if (threadIdx.x == 0) sg.retire = 0;
+  }
+  __syncthreads();
+}
+
+/* slot of the request of rank `rank` in the block's share of class c, and its
+ * segment j; null: not known */
+__device__ __forceinline__ unsigned long long *blk_segs_slot(const ouro_heap_dev &h, const blk_segs &sg, int c,
+                                                             unsigned rank, unsigned &j) {
+  const unsigned off = sg.off0[c] + rank;
+  j = off / h.seg_cap;
+  return j < BLK_SEGS && sg.cells[c][j] ? sg.cells[c][j] + (off - j * h.seg_cap) : nullptr;
+}
+
+/* Counts the block's events and retires the segments that saw their last one.
+ * Called by every thread after a block barrier. */
+template <int QF>
+__device__ void blk_segs_events(const ouro_heap_dev &h, blk_segs &sg) {
+  if (threadIdx.x < OURO_MAX_CLASSES * BLK_SEGS) {
+    const unsigned c = threadIdx.x / BLK_SEGS, j = threadIdx.x % BLK_SEGS, n = sg.events[c][j];
+    if (n) {
+      const unsigned x = (unsigned)(((const unsigned char *)sg.cells[c][j] - h.base) >> h.log2_chunk);
+      if (atomicAdd(&seg_of(h, x)->done, n) + n == 2u * h.seg_cap) {
+        __threadfence();
+        if (QF == OURO_QF_LIST) atomicOr(&sg.retire, 1u << c);
+        else va_retire(h, (int)c, x);
+      }
+    }
+  }
+  if (QF != OURO_QF_LIST) return;
+  __syncthreads();
+  for (unsigned rm = sg.retire, k = 0; rm; rm &= rm - 1, ++k)   /* a warp for each such class */
+    if (k % (blockDim.x >> 5) == threadIdx.x >> 5) vl_advance_warp<OURO_VL_WIDE_BATCH>(h, __ffs(rm) - 1);
+}
+
+/* out of line: R copies of the warp path inlined spilled 2 KB a thread */
+template <int V>
+__device__ __noinline__ void *blk_malloc_rest(const ouro_heap_dev &h, int cls, unsigned long long pos) {
+  return page_malloc<V, 1, true>(h, cls, 0xffffffffu, pos);
+}
+template <int V>
+__device__ __noinline__ void blk_free_rest(const ouro_heap_dev &h, int cls, unsigned item, unsigned vmask,
+                                           unsigned long long pos) {
+  page_free<V, true>(h, cls, item, vmask, pos);
+}
+
 template <int V, int R>
 __global__ void __launch_bounds__(256, 4) k_batch_malloc_blk(ouro_heap_dev h, const uint32_t *sizes, void **ptrs,
                                                              size_t n) {
   ouro::chain_begin();
-  constexpr bool RING = ouro_qform(V) == OURO_QF_RING;
+  constexpr int QF = ouro_qform(V);
+  constexpr bool RING = QF == OURO_QF_RING, SEGS = !RING && R > 1;
+  __shared__ typename std::conditional<SEGS, blk_segs, char>::type sg;
   __shared__ unsigned s_cnt[OURO_MAX_CLASSES], s_ok[OURO_MAX_CLASSES];
   __shared__ unsigned long long s_pos[OURO_MAX_CLASSES];
   __shared__ unsigned long long *s_ring[OURO_MAX_CLASSES];
@@ -94,17 +199,45 @@ __global__ void __launch_bounds__(256, 4) k_batch_malloc_blk(ouro_heap_dev h, co
     __syncthreads();
     blk_reserve<R>(cls, pos, s_cnt);
     __syncthreads();
-    if (threadIdx.x < OURO_MAX_CLASSES && s_cnt[threadIdx.x])
+    if (threadIdx.x < OURO_MAX_CLASSES && s_cnt[threadIdx.x]) {
+      if constexpr (SEGS) sg.end[threadIdx.x] = ld_rlx(&qh(h, threadIdx.x)->tail.v);
       s_pos[threadIdx.x] = atomicAdd(&qh(h, threadIdx.x)->head.v, (unsigned long long)s_cnt[threadIdx.x]);
+    }
     __syncthreads();
     void *res[R];
     bool pend[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-      if (cls[r] >= 0) pos[r] += s_pos[cls[r]];
       res[r] = nullptr;
       pend[r] = cls[r] >= 0;
     }
+    if constexpr (SEGS) {   /* fast path of virtualized queues: every position's slot at once */
+      blk_segs_find<QF, false>(h, sg, s_cnt, s_pos);
+      if (!h.checked) {
+        unsigned long long v[R];
+        unsigned j[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          unsigned long long *cell = pend[r] ? blk_segs_slot(h, sg, cls[r], (unsigned)pos[r], j[r]) : nullptr;
+          v[r] = cell ? ld_rlx(cell) : 0ull;
+          if (!cell) j[r] = BLK_SEGS;
+        }
+        fence_acq_rel();
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          if (!pend[r] || j[r] == BLK_SEGS) continue;
+          const int d = slot_d(v[r], pos[r] + s_pos[cls[r]]);
+          if (d == 1 || d == 2) {
+            if (d == 1) res[r] = blk_block(h, cls[r], lo32(v[r]));
+            atomicAdd(&sg.events[cls[r]][j[r]], 1u);
+            pend[r] = false;
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+      if (cls[r] >= 0) pos[r] += s_pos[cls[r]];
     if (RING && !h.checked) {   /* fast path: every position's slot at once */
       unsigned long long v[R];
 #pragma unroll
@@ -117,14 +250,7 @@ __global__ void __launch_bounds__(256, 4) k_batch_malloc_blk(ouro_heap_dev h, co
         const int d = slot_d(v[r], pos[r]);
         if (d == 1 || d == 2) {   /* an item, or the heap's null answer: take it, retire the slot */
           st_rlx(s_ring[cls[r]] + (pos[r] & s_rmask[cls[r]]), slot(pos[r] + s_rmask[cls[r]] + 1, 0));
-          if (d == 1) {
-            unsigned sh = 4u + cls[r];
-            if (cls[r] >= (int)h.n_classes) {   /* a run: the item is its first chunk, live again */
-              h.chunk_cls[lo32(v[r])] = (unsigned char)cls[r];
-              sh = h.log2_chunk;
-            }
-            res[r] = h.base + ((size_t)lo32(v[r]) << sh);
-          }
+          if (d == 1) res[r] = blk_block(h, cls[r], lo32(v[r]));
           pend[r] = false;
         }
       }
@@ -132,7 +258,9 @@ __global__ void __launch_bounds__(256, 4) k_batch_malloc_blk(ouro_heap_dev h, co
 #pragma unroll
     for (int r = 0; r < R; ++r) {   /* the rest: the warp path from the taken positions */
       if (!__any_sync(0xffffffffu, pend[r])) continue;
-      void *q = page_malloc<V, 1, true>(h, pend[r] ? cls[r] : -1, 0xffffffffu, pos[r]);
+      void *q;
+      if constexpr (SEGS) q = blk_malloc_rest<V>(h, pend[r] ? cls[r] : -1, pos[r]);
+      else q = page_malloc<V, 1, true>(h, pend[r] ? cls[r] : -1, 0xffffffffu, pos[r]);
       if (pend[r]) res[r] = q;
     }
 #pragma unroll
@@ -142,6 +270,7 @@ __global__ void __launch_bounds__(256, 4) k_batch_malloc_blk(ouro_heap_dev h, co
       if (res[r]) atomicAdd(&s_ok[cls[r]], 1u);
     }
     __syncthreads();
+    if constexpr (SEGS) blk_segs_events<QF>(h, sg);
     if (threadIdx.x < OURO_MAX_CLASSES && s_cnt[threadIdx.x]) {
       stat_add(h, threadIdx.x, OURO_ST_MALLOC, s_ok[threadIdx.x]);
       stat_add(h, threadIdx.x, OURO_ST_FAILED, s_cnt[threadIdx.x] - s_ok[threadIdx.x]);
@@ -154,7 +283,9 @@ __global__ void __launch_bounds__(256, 4) k_batch_malloc_blk(ouro_heap_dev h, co
 template <int V, int R>
 __global__ void __launch_bounds__(256) k_batch_free_blk(ouro_heap_dev h, void *const *ptrs, size_t n) {
   ouro::chain_begin();
-  constexpr bool RING = ouro_qform(V) == OURO_QF_RING;
+  constexpr int QF = ouro_qform(V);
+  constexpr bool RING = QF == OURO_QF_RING, SEGS = !RING && R > 1;
+  __shared__ typename std::conditional<SEGS, blk_segs, char>::type sg;
   __shared__ unsigned s_cnt[OURO_MAX_CLASSES];
   __shared__ unsigned long long s_pos[OURO_MAX_CLASSES];
   __shared__ unsigned long long *s_ring[OURO_MAX_CLASSES];
@@ -189,11 +320,33 @@ __global__ void __launch_bounds__(256) k_batch_free_blk(ouro_heap_dev h, void *c
     }
     __syncthreads();
     bool pend[R];
+    if constexpr (SEGS) blk_segs_find<QF, true>(h, sg, s_cnt, s_pos);
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-      if (cls[r] >= 0) pos[r] += s_pos[cls[r]];
-      pend[r] = cls[r] >= 0;
+    for (int r = 0; r < R; ++r) pend[r] = cls[r] >= 0;
+    if constexpr (SEGS) {   /* fast path of virtualized queues: one release fence, then every slot's exchange at once */
+      unsigned long long old[R];
+      unsigned j[R];
+      fence_acq_rel();
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        unsigned long long *cell = pend[r] ? blk_segs_slot(h, sg, cls[r], (unsigned)pos[r], j[r]) : nullptr;
+        if (cell) old[r] = exch_rlx(cell, slot(pos[r] + s_pos[cls[r]] + 1, item[r]));
+        else j[r] = BLK_SEGS;
+      }
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        if (!pend[r] || j[r] == BLK_SEGS) continue;
+        if (slot_d(old[r], pos[r] + s_pos[cls[r]]) >= 3) {   /* its consumer gave the position up */
+          stat_add(h, cls[r], OURO_ST_REPUSH, 1);
+          push_one<QF>(h, cls[r], item[r]);
+        }
+        atomicAdd(&sg.events[cls[r]][j[r]], 1u);
+        pend[r] = false;
+      }
     }
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+      if (cls[r] >= 0) pos[r] += s_pos[cls[r]];
     if (RING) {   /* fast path: one release fence, then every slot's CAS at once */
       unsigned long long old[R];
       fence_acq_rel();
@@ -208,9 +361,15 @@ __global__ void __launch_bounds__(256) k_batch_free_blk(ouro_heap_dev h, void *c
 #pragma unroll
     for (int r = 0; r < R; ++r) {   /* the rest: the warp path at the taken positions */
       const unsigned vmask = __ballot_sync(0xffffffffu, pend[r]);
-      if (pend[r]) page_free<V, true>(h, cls[r], item[r], vmask, pos[r]);
+      if (!pend[r]) continue;
+      if constexpr (SEGS) blk_free_rest<V>(h, cls[r], item[r], vmask, pos[r]);
+      else page_free<V, true>(h, cls[r], item[r], vmask, pos[r]);
     }
     __syncthreads();
+    if constexpr (SEGS) {
+      blk_segs_events<QF>(h, sg);
+      __syncthreads();
+    }
   }
 }
 
@@ -614,10 +773,9 @@ struct pattern_shape {
 namespace ouro {
 namespace launch {
 
-/* Requests per thread of the block-aggregated kernels: four on plain arrays
- * (their slots are tried together) once a batch fills every SM with four
- * per thread; one otherwise, and always on virtualized queues, so that a
- * small batch still spreads over many blocks. */
+/* Requests per thread of the block-aggregated kernels: four (their slots are
+ * tried together) once a batch fills every SM with four per thread; one
+ * otherwise, so that a small batch still spreads over many blocks. */
 constexpr int BLK_WIDE = 4;
 inline bool blk_wide(size_t n) { return n >= (size_t)BLK_WIDE * 256 * ouro::host::sm_count(); }
 /* The plain-array batch free takes eight requests per thread in blocks of
@@ -631,13 +789,11 @@ ouro_status batch_malloc(ouro_heap *H, const uint32_t *d_sizes, void **d_ptrs, s
   const int block = 256;
   if constexpr (ouro_page_queues(V)) {
     if (!H->d.deopt) {
-      if constexpr (ouro_qform(V) == OURO_QF_RING) {
-        if (blk_wide(n)) {
-          ouro::host::launch_chained(k_batch_malloc_blk<V, BLK_WIDE>, grid_for((n + BLK_WIDE - 1) / BLK_WIDE, block, 1 << 20), block, s,
+      if (blk_wide(n)) {
+        ouro::host::launch_chained(k_batch_malloc_blk<V, BLK_WIDE>, grid_for((n + BLK_WIDE - 1) / BLK_WIDE, block, 1 << 20), block, s,
                                        H->d, d_sizes, d_ptrs, n);
-          OURO_LAUNCHED();
-          return OURO_OK;
-        }
+        OURO_LAUNCHED();
+        return OURO_OK;
       }
       ouro::host::launch_chained(k_batch_malloc_blk<V, 1>, grid_for(n, block, 1 << 20), block, s,
                                        H->d, d_sizes, d_ptrs, n);
@@ -674,12 +830,12 @@ ouro_status batch_free(ouro_heap *H, void *const *d_ptrs, size_t n, cudaStream_t
           OURO_LAUNCHED();
           return OURO_OK;
         }
-        if (blk_wide(n)) {
-          ouro::host::launch_chained(k_batch_free_blk<V, BLK_WIDE>, grid_for((n + BLK_WIDE - 1) / BLK_WIDE, block, 1 << 20), block, s,
+      }
+      if (blk_wide(n)) {
+        ouro::host::launch_chained(k_batch_free_blk<V, BLK_WIDE>, grid_for((n + BLK_WIDE - 1) / BLK_WIDE, block, 1 << 20), block, s,
                                        H->d, d_ptrs, n);
-          OURO_LAUNCHED();
-          return OURO_OK;
-        }
+        OURO_LAUNCHED();
+        return OURO_OK;
       }
       ouro::host::launch_chained(k_batch_free_blk<V, 1>, grid_for(n, block, 1 << 20), block, s,
                                        H->d, d_ptrs, n);

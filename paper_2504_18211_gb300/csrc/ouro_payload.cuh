@@ -123,7 +123,7 @@ struct payload_acc {
  * over the whole row of units, four loads in flight per lane: a row of 32
  * blocks of 16 B is one store and one load per lane instead of 32 round
  * trips with 31 lanes idle (3 * 2^18 blocks of 64 B: write 45 -> 17 us, check
- * 88 -> 20 us; a fused round of 10,240 blocks of 16 B 37 -> 12 us).  Larger
+ * 88 -> 20 us; a fused round of 10,240 blocks of 16 B 37 -> 12 us, 11 since).  Larger
  * blocks fill the warp by themselves and go one at a time, so that a block is
  * read back while L2 still holds it (laying all 32 end to end pushed most of
  * the read-back out to DRAM).  The rests are done by the lanes that hold the
