@@ -47,11 +47,13 @@ int sm_count();
  * gets at least four tasks, so that the last ones fill the gaps, of at least
  * eight requests, which share their queue atomics.  On chunk queues the steps
  * that a task's requests share (pop, reserve, claim, queue again) cost more
- * than uneven ends do, so their tasks go up to 32 requests first (200,003
- * requests on the staged virtualized array: tasks of 16 153 us, of 32 140). */
+ * than uneven ends do, so their tasks go up to 32 requests first, with half
+ * of the warps idle if need be (200,003 requests on the staged virtualized
+ * array: tasks of 16 153 us, of 32 140; 30,011 on the chunk array: tasks of 16
+ * 124 us, of 32 105; 3001: tasks of 4 56 us, of 32 80). */
 inline unsigned round_task(unsigned long long n, unsigned long long warps, bool page_queues) {
   unsigned t = 1;
-  while (t < (page_queues ? 8u : 32u) && t * warps < n) t *= 2;
+  while (t < (page_queues ? 8u : 32u) && t * warps < (page_queues ? n : 2 * n)) t *= 2;
   while (t < 32 && 8 * t * warps <= n) t *= 2;
   return t;
 }

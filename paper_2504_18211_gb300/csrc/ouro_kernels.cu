@@ -473,7 +473,7 @@ __global__ void __launch_bounds__(256) k_batch_free_cblk(ouro_heap_dev h, void *
  * of them runs that each went through the warp path, malloc to free: 105 us, 94
  * with this and the free above.) */
 template <int V, int R>
-__global__ void __launch_bounds__(256, 2) k_batch_malloc_cblk(ouro_heap_dev h, const uint32_t *sizes, void **ptrs,
+__global__ void __launch_bounds__(256) k_batch_malloc_cblk(ouro_heap_dev h, const uint32_t *sizes, void **ptrs,
                                                            size_t n) {
   ouro::chain_begin();
   constexpr bool RING = ouro_qform(V) == OURO_QF_RING;
