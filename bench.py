@@ -79,8 +79,8 @@ def dist_env():
 # from the sources whose digest is recorded; null once they change.
 FUSED_KERNEL_SOURCES = ("include/ouro_device.cuh", "paper_2504_18211_gb300/csrc/ouro_payload.cuh",
                         "paper_2504_18211_gb300/csrc/ouro_kernels.cu", "paper_2504_18211_gb300/csrc/ouro_internal.cuh")
-FUSED_TRAFFIC = {"sources_sha256": "ca166ebb2bafe0ca9cfc517fc553e8fb6b8e82b85de8608ef8652ec590515386",
-                 "bytes_per_launch": 1643345152}
+FUSED_TRAFFIC = {"sources_sha256": "85164d140b152eaef28e2ab7c0c0768d169632a415cdf4cad08cb7d105bfaf20",
+                 "bytes_per_launch": 1712762624}
 
 
 def kernel_sources_digest() -> str:
