@@ -79,7 +79,7 @@ def dist_env():
 # from the sources whose digest is recorded; null once they change.
 FUSED_KERNEL_SOURCES = ("include/ouro_device.cuh", "paper_2504_18211_gb300/csrc/ouro_payload.cuh",
                         "paper_2504_18211_gb300/csrc/ouro_kernels.cu", "paper_2504_18211_gb300/csrc/ouro_internal.cuh")
-FUSED_TRAFFIC = {"sources_sha256": "85164d140b152eaef28e2ab7c0c0768d169632a415cdf4cad08cb7d105bfaf20",
+FUSED_TRAFFIC = {"sources_sha256": "b6d318d33dc47e98b48fd21ef45a0f22d6c46f739402f37394cde5fd49474338",
                  "bytes_per_launch": 1712762624}
 
 

@@ -470,7 +470,7 @@ __global__ void __launch_bounds__(256) k_batch_free_cblk(ouro_heap_dev h, void *
  * block too; on plain arrays a thread tries all its runs' slots together, and
  * what is not ready takes the warp path of page_malloc at the position already
  * taken.  Statistics once per class per block.  (300,007 mixed requests, 2 %
- * of them runs that each went through the warp path, malloc to free: 105 us, 94
+ * of them runs that each went through the warp path, malloc to free: 105 us, 98
  * with this and the free above.) */
 template <int V, int R>
 __global__ void __launch_bounds__(256) k_batch_malloc_cblk(ouro_heap_dev h, const uint32_t *sizes, void **ptrs,
