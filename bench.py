@@ -79,7 +79,7 @@ def dist_env():
 # from the sources whose digest is recorded; null once they change.
 FUSED_KERNEL_SOURCES = ("include/ouro_device.cuh", "paper_2504_18211_gb300/csrc/ouro_payload.cuh",
                         "paper_2504_18211_gb300/csrc/ouro_kernels.cu", "paper_2504_18211_gb300/csrc/ouro_internal.cuh")
-FUSED_TRAFFIC = {"sources_sha256": "b6d318d33dc47e98b48fd21ef45a0f22d6c46f739402f37394cde5fd49474338",
+FUSED_TRAFFIC = {"sources_sha256": "8fd89ca53171beef4b24fce5813c76db6a7e924fe5ec6114411f268fae08ce19",
                  "bytes_per_launch": 1712762624}
 
 

@@ -385,7 +385,7 @@ __global__ void __launch_bounds__(256) k_batch_free_blk(ouro_heap_dev h, void *c
  * filled behind one fence; a slot that is not ready, and the slots of
  * virtualized queues, take the warp path at the position already taken.
  * Statistics once per class per block.  (300,007 mixed requests, 2 % of them
- * runs that each went through the warp path, malloc to free: 105 us, 94 with
+ * runs that each went through the warp path, malloc to free: 105 us, 98 with
  * this and the malloc below.) */
 template <int V, int R>
 __global__ void __launch_bounds__(256) k_batch_free_cblk(ouro_heap_dev h, void *const *ptrs, size_t n) {
