@@ -240,8 +240,10 @@ ouro_status ouro_pattern_check(void *const *d_ptrs, const uint32_t *d_sizes, siz
                                uint32_t seed, int mode, ouro_check *d_out, void *stream);
 
 /* One whole driver round in ONE kernel: every request allocates, writes its
- * pattern, reads it back and frees.  *d_out (device) receives the check.
- * d_ptrs (device, optional): receives each request's block address. */
+ * pattern, reads it back and frees.  *d_out (device) receives the check; it
+ * belongs to the round until it has finished.  d_ptrs (device, optional):
+ * receives each request's block address.  Rounds on one heap may be in flight
+ * on any number of streams and in replayed graphs at once. */
 ouro_status ouro_round_fused(ouro_heap *h, const uint32_t *d_sizes, size_t n, uint32_t seed,
                              int mode, ouro_check *d_out, void **d_ptrs, void *stream);
 

@@ -161,7 +161,36 @@ struct ouro_batch_graph {
   cudaGraphExec_t exec;
   size_t nodes;
   size_t kernels;   /* kernel nodes: the library's launches per replay */
+  void *work;       /* its rounds' work slot; null: they work in their results (no memory for a slot) */
 };
+
+/* The graph's own work slot, zero: its rounds are one chain and a graph never
+ * runs beside itself, so they share it.  Null where there is no memory for it.
+ * Another thread may be capturing: nothing here touches its streams. */
+static void *graph_work(cudaStream_t s) {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  void *work = nullptr;
+  if (cudaMalloc(&work, 128) != cudaSuccess) {
+    cudaGetLastError();
+    work = nullptr;
+  } else if (cudaMemsetAsync(work, 0, 128, s) != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess) {
+    cudaGetLastError();
+    cudaFree(work);
+    work = nullptr;
+  }
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  return work;
+}
+
+/* waits for the replays in flight */
+static void graph_work_free(void *work) {
+  if (!work) return;
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  cudaFree(work);
+  cudaThreadExchangeStreamCaptureMode(&mode);
+}
 
 extern "C" ouro_status ouro_batches_persistent(ouro_heap *H, const uint32_t *d_sizes, const unsigned long long *d_offs,
                                                const unsigned long long *d_task_offs, uint32_t n_batches,
@@ -197,13 +226,16 @@ extern "C" ouro_status ouro_batch_graph_create(ouro_heap *H, const uint32_t *d_s
                                                void **d_ptrs, int form, ouro_batch_graph **out) {
   if (!H || !d_sizes || !h_offs || !d_out || !out || n_batches == 0 || (form == 1 && !d_ptrs) || form < 0 || form > 1)
     return OURO_EINVAL;
+  if (mode != 0 && mode != 1) return OURO_EINVAL;
   *out = nullptr;
   cudaStream_t cs;
   OURO_CUDA(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
   ouro_status st = OURO_OK;
   cudaGraph_t g = nullptr;
+  void *work = form == 0 ? graph_work(cs) : nullptr;
   cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
   if (e != cudaSuccess) {
+    graph_work_free(work);
     cudaStreamDestroy(cs);
     return ouro::host::cuda_fail(e);
   }
@@ -211,7 +243,7 @@ extern "C" ouro_status ouro_batch_graph_create(ouro_heap *H, const uint32_t *d_s
     const size_t n = (size_t)(h_offs[b + 1] - h_offs[b]);
     const uint32_t *sz = d_sizes + h_offs[b];
     if (form == 0) {
-      st = ouro_round_fused(H, sz, n, seed + b, mode, d_out + b, nullptr, cs);
+      st = ouro::host::round_fused_on(H, sz, n, seed + b, mode, d_out + b, nullptr, work, cs);
     } else {
       st = ouro_batch_malloc(H, sz, d_ptrs, n, cs);
       if (st == OURO_OK) st = ouro_pattern_write(d_ptrs, sz, n, seed + b, mode, cs);
@@ -223,7 +255,7 @@ extern "C" ouro_status ouro_batch_graph_create(ouro_heap *H, const uint32_t *d_s
   if (st == OURO_OK && e != cudaSuccess) st = ouro::host::cuda_fail(e);
   ouro_batch_graph *G = nullptr;
   if (st == OURO_OK) {
-    G = new ouro_batch_graph{g, nullptr, 0, 0};
+    G = new ouro_batch_graph{g, nullptr, 0, 0, work};
     e = cudaGraphInstantiate(&G->exec, g, 0);
     if (e != cudaSuccess) st = ouro::host::cuda_fail(e);
     cudaGraphGetNodes(g, nullptr, &G->nodes);
@@ -241,6 +273,7 @@ extern "C" ouro_status ouro_batch_graph_create(ouro_heap *H, const uint32_t *d_s
       delete G;
     }
     if (g) cudaGraphDestroy(g);
+    graph_work_free(work);
     return st;
   }
   *out = G;
@@ -260,6 +293,7 @@ extern "C" ouro_status ouro_batch_graph_destroy(ouro_batch_graph *G) {
   if (!G) return OURO_OK;
   cudaGraphExecDestroy(G->exec);
   cudaGraphDestroy(G->graph);
+  graph_work_free(G->work);
   delete G;
   return OURO_OK;
 }

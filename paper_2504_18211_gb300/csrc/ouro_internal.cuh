@@ -14,8 +14,8 @@
 /* virtualized-array directories also span positions that are waiting for a
  * producer or in flight (more than twice the resident threads of 152 SMs) */
 #define OURO_VA_SLACK (1ull << 20)
-/* work slots of fused rounds: one per launch in flight on a heap, each on its
- * own 128-byte line, handed out round robin; zero between launches */
+/* work slots of fused rounds: one per stream that launches them on a heap (up
+ * to this many), each on its own 128-byte line; zero between launches */
 #define OURO_WORK_SLOTS 64
 
 struct ouro_heap {
@@ -26,7 +26,7 @@ struct ouro_heap {
   unsigned char *meta;          /* one device allocation for every metadata table */
   size_t meta_bytes;
   size_t off_qhdr, off_glob, off_stats, off_cls, off_pool, off_free, off_bits, off_cells, off_work;
-  unsigned work_seq;            /* next work-counter slot (atomic) */
+  unsigned long long work_stream[OURO_WORK_SLOTS];   /* stream that slot k belongs to: its id + 1; 0: none (atomic) */
   size_t stats_words;
   unsigned long long ring_total;
   ouro_options opt;
@@ -38,6 +38,9 @@ extern thread_local int g_last_cuda_error;
 ouro_status cuda_fail(cudaError_t e);
 void count_launch(unsigned n = 1);
 int sm_count();
+/* ouro_round_fused, its arguments checked, with a given work slot (null: none) */
+ouro_status round_fused_on(ouro_heap *H, const uint32_t *d_sizes, size_t n, uint32_t seed, int mode, ouro_check *d_out,
+                           void **d_ptrs, void *work, cudaStream_t s);
 
 /* Requests that a warp of the fused kernels takes at a time, 2^0 .. 2^5, for
  * n requests on `warps` resident warps.  A warp walks its larger blocks one

@@ -664,11 +664,26 @@ __global__ void __launch_bounds__(256) k_pattern(void *const *ptrs, const uint32
   if (OP & PAY_CHECK) flush_acc(a, nulls, out);
 }
 
+/* A fused round's tasks past the warps' first ones: drawn from a counter in the
+ * launch's slot, or without one in the half of *out's xor64 that stays zero. */
+struct round_draws {
+  unsigned long long first = 0;   /* the first request that is drawn for */
+  unsigned *next;
+  unsigned count = 0;             /* draws in all; 0: none */
+  round_draws(size_t n, unsigned task, unsigned warps, work_slot *work, ouro_check *out) {
+    first = (unsigned long long)warps * task;
+    if (first < n) count = (unsigned)((n - first + task - 1) / task) + warps;
+    next = work ? &work->next : reinterpret_cast<unsigned *>(&out->xor64) + 1;
+  }
+};
+
 /* one whole round per thread: malloc, write, read back, free.  Warps take
  * `task` requests (a power of two of at most 32) at a time: warp w of the
- * grid the w-th task, then tasks from the launch's work slot, so blocks of
+ * grid the w-th task, then tasks from the launch's counter, so blocks of
  * uneven sizes balance across warps and the round ends within one task of
- * the last byte.  The lanes past `task` ask for nothing but help their
+ * the last byte.  Where tasks are drawn at all, every warp draws until there
+ * is none left, so the number of draws is known and the last one leaves the
+ * counter zero.  The lanes past `task` ask for nothing but help their
  * warp's carves and payload.  STAGE: the warp's freed pages serve its next
  * mallocs of the same class from shared memory (heap option `staging`). */
 #ifndef OURO_FUSED_MIN_BLOCKS
@@ -679,14 +694,13 @@ __global__ void __launch_bounds__(256) k_pattern(void *const *ptrs, const uint32
 template <int V, bool STAGE>
 __global__ void __launch_bounds__(256, ouro_page_queues(V) ? OURO_FUSED_MIN_BLOCKS : 2) k_round_fused(ouro_heap_dev h, const uint32_t *sizes, size_t n,
                                                      uint32_t seed, int mode, unsigned task, ouro_check *out,
-                                                     void **ptrs, work_slot *work) {
+                                                     void **ptrs, work_slot *work, round_draws draw) {
   ouro::chain_begin();
   __shared__ ouro_block_ctx<8> ctx;
   if (STAGE) ouro_block_begin(ctx);
   payload_acc a;
   unsigned long long nulls = 0;
   const unsigned lane = threadIdx.x & 31;
-  const unsigned long long first = (unsigned long long)gridDim.x * (blockDim.x >> 5) * task;   /* tasks not handed out */
   unsigned long long base = (unsigned long long)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * task;
   while (base < n) {
     const size_t i = base + lane;
@@ -707,8 +721,12 @@ __global__ void __launch_bounds__(256, ouro_page_queues(V) ? OURO_FUSED_MIN_BLOC
     if (STAGE) ouro::detail::stage_free<V, 8>(ctx, h, p, __activemask(), p ? size_class(h, sz) : -1);
     else free_v<V>(h, p);
     __syncwarp();
-    if (first >= n) break;
-    if (lane == 0) base = first + atomicAdd(&work->next, (unsigned long long)task);
+    if (!draw.count) break;
+    if (lane == 0) {
+      const unsigned d = atomicAdd(draw.next, 1u);
+      base = draw.first + (unsigned long long)d * task;
+      if (d == draw.count - 1) *draw.next = 0;
+    }
     base = __shfl_sync(0xffffffffu, base, 0);
   }
   if (STAGE) ouro_block_end_v<V>(ctx, h);
@@ -865,8 +883,10 @@ ouro_status round_fused_form(ouro_heap *H, const uint32_t *d_sizes, size_t n, ui
                              ouro_check *d_out, void **d_ptrs, void *work, cudaStream_t s) {
   const int block = 256, cap = occupancy_grid(k_round_fused<V, STAGE>, block);
   const unsigned task = ouro::host::round_task(n, (size_t)cap * (block / 32), ouro_page_queues(V));
-  ouro::host::launch_chained(k_round_fused<V, STAGE>, grid_for((n + task - 1) / task * 32, block, cap), block, s,
-                             H->d, d_sizes, n, seed, mode, task, d_out, d_ptrs, static_cast<work_slot *>(work));
+  const int grid = grid_for((n + task - 1) / task * 32, block, cap);
+  work_slot *slot = static_cast<work_slot *>(work);
+  ouro::host::launch_chained(k_round_fused<V, STAGE>, grid, block, s, H->d, d_sizes, n, seed, mode, task, d_out,
+                             d_ptrs, slot, round_draws(n, task, grid * (block / 32), slot, d_out));
   OURO_LAUNCHED();
   return OURO_OK;
 }
@@ -932,19 +952,55 @@ extern "C" ouro_status ouro_pattern_check(void *const *d_ptrs, const uint32_t *d
   return OURO_OK;
 }
 
+namespace ouro {
+namespace host {
+ouro_status round_fused_on(ouro_heap *H, const uint32_t *d_sizes, size_t n, uint32_t seed, int mode, ouro_check *d_out,
+                           void **d_ptrs, void *work, cudaStream_t s) {
+  if (!n || !work) OURO_CUDA(cudaMemsetAsync(d_out, 0, sizeof(ouro_check), s));
+  if (!n) return OURO_OK;
+  OURO_DISPATCH(H->d.variant, return ouro::launch::round_fused<V>(H, d_sizes, n, seed, mode, d_out, d_ptrs, work, s));
+}
+
+/* The work slot of an eager round on stream s; null (the round then works in
+ * its own zeroed result) for a round that is being captured, and where all
+ * slots belong to other streams.  A slot belongs to one stream for the heap's
+ * life: the launches of a stream run one after another, so no two launches
+ * meet on it, however many are in flight and however long one takes.  Streams
+ * are told apart by their ids, which are not used again when a stream is
+ * destroyed.  A captured round has no such order: its graph may be replayed
+ * beside anything, from any stream.  The entries of the table only ever go
+ * from 0 to an id, first free entry first, so a stream never gets two. */
+static ouro_status round_work(ouro_heap *H, cudaStream_t s, void **work) {
+  *work = nullptr;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  OURO_CUDA(cudaStreamIsCapturing(s, &cap));
+  if (cap != cudaStreamCaptureStatusNone) return OURO_OK;
+  unsigned long long id = 0;
+  OURO_CUDA(cudaStreamGetId(s, &id));
+  ++id;   /* 0 marks a free entry */
+  for (unsigned k = 0; k < OURO_WORK_SLOTS; ++k) {
+    unsigned long long have = __atomic_load_n(&H->work_stream[k], __ATOMIC_RELAXED);
+    if (!have && __atomic_compare_exchange_n(&H->work_stream[k], &have, id, false, __ATOMIC_RELAXED, __ATOMIC_RELAXED))
+      have = id;
+    if (have == id) {
+      *work = H->meta + H->off_work + (size_t)k * 128;
+      break;
+    }
+  }
+  return OURO_OK;
+}
+}  // namespace host
+}  // namespace ouro
+
 extern "C" ouro_status ouro_round_fused(ouro_heap *H, const uint32_t *d_sizes, size_t n, uint32_t seed, int mode,
                                         ouro_check *d_out, void **d_ptrs, void *stream) {
   if (!H || !d_out || (n && !d_sizes)) return OURO_EINVAL;
   if (mode != 0 && mode != 1) return OURO_EINVAL;
-  if (!n) {
-    OURO_CUDA(cudaMemsetAsync(d_out, 0, sizeof(ouro_check), S(stream)));
-    return OURO_OK;
+  void *work = nullptr;
+  if (n) {
+    const ouro_status st = ouro::host::round_work(H, S(stream), &work);
+    if (st != OURO_OK) return st;
   }
-  /* this launch's work slot, one of the heap's ring (launches in flight at
-   * once on one heap: up to 64); the launch leaves it zero */
-  const unsigned slot = __atomic_fetch_add(&H->work_seq, 1u, __ATOMIC_RELAXED) % OURO_WORK_SLOTS;
-  void *work = H->meta + H->off_work + (size_t)slot * 128;
-  OURO_DISPATCH(H->d.variant,
-                return ouro::launch::round_fused<V>(H, d_sizes, n, seed, mode, d_out, d_ptrs, work, S(stream)));
+  return ouro::host::round_fused_on(H, d_sizes, n, seed, mode, d_out, d_ptrs, work, S(stream));
 }
 #endif

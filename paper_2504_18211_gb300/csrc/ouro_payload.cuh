@@ -357,32 +357,39 @@ __device__ inline void block_acc(payload_acc &a, unsigned long long nulls, unsig
   __syncthreads();
 }
 
-/* the block's check counters added to *out (zero when the kernel began) */
+/* A block's counters (block_acc) added to *out, which was zero when the
+ * kernel began.  The words are 32-bit, so their XOR only ever touches the low
+ * half of xor64; the high half may hold a fused round's task counter. */
+__device__ __forceinline__ void add_check(const unsigned long long (&sm)[5], ouro_check *out) {
+  if (sm[0]) atomicAdd(&out->nulls, sm[0]);
+  if (sm[1]) atomicAdd(&out->mismatches, sm[1]);
+  atomicXor(reinterpret_cast<unsigned *>(&out->xor64), (unsigned)sm[2]);
+  atomicAdd(&out->sum64, sm[3]);
+  atomicAdd(&out->words, sm[4]);
+}
+
 __device__ inline void flush_acc(payload_acc &a, unsigned long long nulls, ouro_check *out) {
   __shared__ unsigned long long sm[5];
   block_acc(a, nulls, sm);
-  if (threadIdx.x == 0) {
-    if (sm[0]) atomicAdd(&out->nulls, sm[0]);
-    if (sm[1]) atomicAdd(&out->mismatches, sm[1]);
-    atomicXor(&out->xor64, sm[2]);
-    atomicAdd(&out->sum64, sm[3]);
-    atomicAdd(&out->words, sm[4]);
-  }
+  if (threadIdx.x == 0) add_check(sm, out);
 }
 
-/* One launch's work slot (a 128-byte line of the heap's metadata): all zero
- * between launches.  The blocks add their counters to acc; the last one to
- * finish writes the sums to *out and leaves the slot zero for the next
- * launch, so a launch needs no memset of its counters or its result. */
+/* A work slot (a 128-byte line): all zero between launches, and never used by
+ * two launches at a time (who may use which: round_work in ouro_kernels.cu).
+ * The blocks add their counters to acc; the last one to finish writes the
+ * sums to *out and leaves the slot zero for the next launch, so a launch needs
+ * no memset of its counters or its result.  A launch without a slot (null)
+ * has *out zeroed before it begins, and adds to that. */
 struct work_slot {
-  unsigned long long next;     /* requests handed out past the warps' first tasks */
+  unsigned next, pad;          /* tasks drawn; zero again after the last draw */
   unsigned long long acc[5];   /* nulls, mismatches, xor, sum, words */
   unsigned long long done;     /* blocks finished */
 };
 __device__ inline void finish_acc(payload_acc &a, unsigned long long nulls, work_slot *w, ouro_check *out) {
   __shared__ unsigned long long sm[5];
   block_acc(a, nulls, sm);
-  if (threadIdx.x == 0) {
+  if (threadIdx.x == 0 && !w) add_check(sm, out);
+  if (threadIdx.x == 0 && w) {
     if (sm[0]) atomicAdd(&w->acc[0], sm[0]);
     if (sm[1]) atomicAdd(&w->acc[1], sm[1]);
     atomicXor(&w->acc[2], sm[2]);
@@ -400,7 +407,6 @@ __device__ inline void finish_acc(payload_acc &a, unsigned long long nulls, work
         o[k] = r[k];
         w->acc[k] = 0;
       }
-      w->next = 0;
       w->done = 0;
     }
   }
