@@ -168,7 +168,7 @@ __device__ void warp_append(const ouro_heap_dev &h, vertex *vx, const unsigned *
       }
       progress |= grow;
       __syncwarp();
-      free_v<V>(h, reinterpret_cast<void *>(old), old ? size_class(h, 4ull * cap) : -1);
+      free_v<V>(h, reinterpret_cast<void *>(old));
       __syncwarp();
     }
 
@@ -341,8 +341,7 @@ k_graph_insert(ouro_heap_dev h, vertex *vt, const unsigned *src, const unsigned 
  * of them for a list of 175,000 entries, which one warp alone copied in 1.3
  * ms (2^22 entries of 2^18 vertices: 1380 us so, 270 with the block, and less
  * with its loads in flight past the ragged end of a segment, whose remainder
- * loop had cost two of its threads seven round trips a segment; that and the
- * free below took init, insert, gather, free and a sort from 1773 to 1593). */
+ * loop had cost two of its threads seven round trips a segment). */
 __global__ void __launch_bounds__(256) k_graph_gather(const vertex *vt, unsigned nv, const unsigned long long *off,
                                                       unsigned *out, unsigned chunk_bytes) {
   constexpr unsigned WARPS = 8;
@@ -393,27 +392,28 @@ __global__ void __launch_bounds__(256) k_graph_gather(const vertex *vt, unsigned
   }
 }
 
-/* Frees every list.  A lane per vertex; the classes are known from the record,
- * so no free reads the chunk table, and a segment's link is read before the
- * frees of the segment before it wait for their queue slots. */
+/* Frees every list.  A lane per vertex; a segment's link is read before the
+ * frees of the segment before it wait for their queue slots.  The classes are
+ * in the records too, but the frees look every block up in the chunk table: a
+ * table from before a reset of the heap, or of another heap, records bad frees
+ * and leaves the queues alone. */
 template <int V>
 __global__ void k_graph_free(ouro_heap_dev h, vertex *vt, unsigned nv) {
   const unsigned threads = gridDim.x * blockDim.x;
   for (unsigned v0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31u); v0 < nv; v0 += threads) {
     const unsigned v = v0 + (threadIdx.x & 31);
-    unsigned long long ptr = 0, seg = 0, end = 0;
+    unsigned long long ptr = 0, seg = 0;
     if (v < nv) {
       ptr = vt[v].ptr;
       seg = vt[v].ovf;
-      end = vt[v].end;
     }
     unsigned long long next = seg ? *reinterpret_cast<const unsigned long long *>(seg) : 0;
     __syncwarp();
-    free_v<V>(h, reinterpret_cast<void *>(ptr), size_class(h, seg ? h.chunk_bytes : 4ull * hi32(end)));
+    free_v<V>(h, reinterpret_cast<void *>(ptr));
     for (unsigned guard = 0; __any_sync(0xffffffffu, seg != 0) && guard < (1u << 26); ++guard) {
       const unsigned long long after = next ? *reinterpret_cast<const unsigned long long *>(next) : 0;
       __syncwarp();
-      free_v<V>(h, reinterpret_cast<void *>(seg), (int)h.n_classes - 1);
+      free_v<V>(h, reinterpret_cast<void *>(seg));
       __syncwarp();
       seg = next;
       next = after;
