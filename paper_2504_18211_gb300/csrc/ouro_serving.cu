@@ -175,7 +175,8 @@ struct serve_lane {
 /* keep (shared memory, one entry per lane of the first warp; null in the
  * per-launch form): the block's sessions stay there from step to step, for
  * grids that hold every slot at once, instead of being read back from memory
- * (two dependent L2 round trips a step). */
+ * (two dependent L2 round trips a step).  k_serve writes those that are still
+ * growing back when it ends. */
 template <int V>
 __device__ void serve_grow(const serve_args &A, uint32_t step, serve_lane *keep) {
   __shared__ unsigned char *s_bp[32];
@@ -375,12 +376,21 @@ __global__ void __launch_bounds__(256, 2) k_serve(serve_args A) {
   for (uint32_t step = 0; step < A.steps; ++step) {
     if (stamps) A.step_ns[3 * step] = globaltimer();
     serve_grow<V>(A, step, keep);
-    if (!grid_barrier(A.ctl, gridDim.x, A.spin_limit, epoch)) return;
+    if (!grid_barrier(A.ctl, gridDim.x, A.spin_limit, epoch)) break;
     if (stamps) A.step_ns[3 * step + 1] = globaltimer();
     if (step + 1 < A.steps) serve_admit(A, step + 1);
     serve_free<V>(A, step);
-    if (!grid_barrier(A.ctl, gridDim.x, A.spin_limit, epoch)) return;
+    if (!grid_barrier(A.ctl, gridDim.x, A.spin_limit, epoch)) break;
     if (stamps) A.step_ns[3 * step + 2] = globaltimer();
+  }
+  if (keep && threadIdx.x < 32 && keep[threadIdx.x].sess >= 0) {   /* unfinished: the caller finds what still lives */
+    const serve_lane &l = keep[threadIdx.x];
+    const unsigned long long slot = blockIdx.x + (unsigned long long)threadIdx.x * gridDim.x;
+    A.slot_session[slot] = l.sess;
+    A.slot_k[slot] = l.k;
+    A.slot_acc[3 * slot] = l.x;
+    A.slot_acc[3 * slot + 1] = l.sum;
+    A.slot_acc[3 * slot + 2] = l.mism;
   }
 }
 
