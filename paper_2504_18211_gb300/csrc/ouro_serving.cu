@@ -30,6 +30,7 @@
  */
 #include <algorithm>
 
+#include "ouro_barrier.cuh"
 #include "ouro_internal.cuh"
 #include "ouro_payload.cuh"
 #include "ouro_shard.cuh"
@@ -69,37 +70,6 @@ __device__ __forceinline__ unsigned long long globaltimer() {
   unsigned long long t;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
   return t;
-}
-
-/* Grid barrier for a cooperative launch: ctl[0] counts arrivals and is never
- * reset, the e-th barrier waits until it reaches e * nblocks, so an arrival is
- * one fence and one atomic, and the wait polls that same word.  A wait that
- * runs out sets ctl[4] and BARRIER_FAILED in the count, which ends every other
- * block's wait. */
-constexpr unsigned long long BARRIER_FAILED = 1ull << 62;
-
-__device__ bool grid_barrier(unsigned long long *ctl, unsigned nblocks, unsigned limit, unsigned &epoch) {
-  __shared__ int ok;
-  __syncthreads();
-  ++epoch;
-  if (threadIdx.x == 0) {
-    const unsigned long long target = (unsigned long long)nblocks * epoch;
-    __threadfence();
-    unsigned long long seen = atomicAdd(&ctl[0], 1ull) + 1;
-    if (seen >= target) __threadfence();
-    for (unsigned it = 0; seen < target; seen = ld_acq(&ctl[0])) {
-      if (++it > limit) {
-        atomicExch(&ctl[4], 1ull);
-        atomicAdd(&ctl[0], BARRIER_FAILED);
-        seen = BARRIER_FAILED;
-        break;
-      }
-      __nanosleep(32);
-    }
-    ok = seen < BARRIER_FAILED;
-  }
-  __syncthreads();
-  return ok != 0;
 }
 
 /* ---------------------------------------------------------------- phases
@@ -517,7 +487,7 @@ ouro_status serve_prepare(ouro_heap *H, const uint32_t *d_arrive_step, const uin
   A.seed = seed;
   A.cap_blocks = cap_blocks;
   A.block_bytes = block_bytes;
-  A.spin_limit = 1u << 24;   /* barrier wait: ~2 s of 128 ns naps, far above any step */
+  A.spin_limit = 1u << 24;   /* barrier wait: each poll is a 32 ns nap and an L2 round trip, seconds in all */
   return OURO_OK;
 }
 }  // namespace
