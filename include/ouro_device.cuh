@@ -1064,6 +1064,39 @@ __device__ __forceinline__ unsigned long long *vl_slot(const ouro_heap_dev &h, i
   return vl_slot_walk(h, c, pos, create);
 }
 
+/* The list's last segment is cur, and the caller has claimed its empty link:
+ * sets the next segment up and links it; its chunk, or NIL where the heap has
+ * none (the link stays claimed).  Behind it, published with the same store,
+ * go up to OURO_VL_RUN - 1 segments of the spare stack, at most OURO_AHEAD_POS
+ * positions past the tail like those that a retire appends.  Retires that find
+ * the link claimed leave their segments on that stack, so a list that has
+ * fallen behind its producers stays there, each segment made on demand while
+ * thousands of warps wait for it.  Fused rounds of 2^20 requests on a list, one
+ * segment at a time and so: any size up to 600 B 2033 and 260 us, 64 B staged
+ * 3750 and 300, 64 B unstaged and not paced (payload_paced) 6300 and 1290; the
+ * rounds that carve a cold list 5.4 ms and 1.6. */
+static __device__ __noinline__ unsigned vl_create_run(const ouro_heap_dev &h, int c, unsigned long long cur) {
+  ouro_qhdr *q = qh(h, c);
+  const unsigned idx = hi32(cur) + 1;
+  const unsigned long long lim = (ld_rlx(&q->tail.v) + OURO_AHEAD_POS) / h.seg_cap;
+  unsigned xs[OURO_VL_RUN], k = 1;
+  xs[0] = seg_new(h, c, idx);
+  if (xs[0] == OURO_NIL) return OURO_NIL;
+  for (; k < OURO_VL_RUN && idx + k <= lim; ++k) {
+    const unsigned x = spare_pop(h, c);
+    if (x == OURO_NIL) break;
+    seg_setup(h, x, idx + k, false, OURO_NIL);
+    seg_of(h, xs[k - 1])->link = pack(idx + k - 1, x);
+    xs[k] = x;
+  }
+  __threadfence();
+  st_rel(&seg_of(h, lo32(cur))->link, pack(hi32(cur), xs[0]));
+  atomicMax(&q->back.v, pack(idx + k - 1, xs[k - 1]));   /* indices only grow */
+  for (unsigned j = 0; j < k; ++j)
+    st_rlx(&q->hint[(idx + j) & (OURO_VL_HINTS - 1)], pack(idx + j, xs[j]));
+  return xs[0];
+}
+
 /* the lookup past a missed hint: out of line, it is the slow path */
 static __device__ __noinline__ unsigned long long *vl_slot_walk(const ouro_heap_dev &h, int c, unsigned long long pos,
                                                         bool create) {
@@ -1124,15 +1157,18 @@ static __device__ __noinline__ unsigned long long *vl_slot_walk(const ouro_heap_
     if (nxt == OURO_NIL) {
       if (!create) return nullptr;
       if (cas_ar(&sg->link, link, pack(hi32(cur), OURO_BUSY)) == link) {
-        unsigned x = seg_new(h, c, hi32(cur) + 1);
+        const bool pages = ouro_page_queues((int)h.variant);
+        const unsigned x = pages ? vl_create_run(h, c, cur) : seg_new(h, c, hi32(cur) + 1);
         if (x == OURO_NIL) {
           st_rel(&sg->link, link);
           set_error(h, OURO_ERR_QUEUE_FULL, OURO_SITE_VL_NEXT);
           return nullptr;
         }
-        st_rel(&sg->link, pack(hi32(cur), x));
         const unsigned long long nb = pack(hi32(cur) + 1, x);
-        cas_ar(&q->back.v, cur, nb);
+        if (!pages) {
+          st_rel(&sg->link, pack(hi32(cur), x));
+          cas_ar(&q->back.v, cur, nb);
+        }
         __threadfence();
         vl_advance(h, c);
         cur = nb;

@@ -85,7 +85,7 @@ k_batches_persistent(ouro_heap_dev h, const uint32_t *sizes, const unsigned long
     else p = static_cast<unsigned char *>(malloc_v<V>(h, sz, active));
     if (active && !p) nulls++;
     __syncwarp();
-    warp_payload<PAY_FUSED>(p, sz, (uint32_t)i, seed + b, mode, a);
+    warp_payload<PAY_FUSED, pace_payload(V, STAGE)>(p, sz, (uint32_t)i, seed + b, mode, a, round_log >= 4);
     __syncwarp();
     if (STAGE) ouro::detail::stage_free<V, 8>(ctx, h, p, __activemask(), p ? size_class(h, sz) : -1);
     else free_v<V>(h, p);

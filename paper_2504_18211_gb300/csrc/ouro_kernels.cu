@@ -714,7 +714,7 @@ __global__ void __launch_bounds__(256, ouro_page_queues(V) ? OURO_FUSED_MIN_BLOC
       if (ptrs) ptrs[i] = p;
     }
     __syncwarp();
-    warp_payload<PAY_FUSED>(p, sz, (uint32_t)i, seed, mode, a);
+    warp_payload<PAY_FUSED, pace_payload(V, STAGE)>(p, sz, (uint32_t)i, seed, mode, a, task >= 16);
     __syncwarp();
     /* staged: the class of each block is known here, so the free skips the
      * chunk-table lookup (one L2 round trip per task off the warp's chain) */

@@ -271,9 +271,44 @@ __device__ __noinline__ payload_acc payload_row(unsigned char *p, uint32_t size,
   return a;
 }
 
-template <int OP>
+/* The blocks one after another, each written and read back through L2 before
+ * the next (OP as above, FUSED only).  Virtualized lists: a warp that holds
+ * its small blocks for the few microseconds of a row takes and gives back
+ * queue positions faster than the list's segments, retired in order, come
+ * round again, and the queue then holds most of the pages and with them most
+ * of the segments (fused rounds of 2^20 requests of 64 B 1290 us, 212 so). */
+__device__ __noinline__ inline payload_acc payload_paced(unsigned char *p, uint32_t size, uint32_t key) {
+  constexpr unsigned FULL = 0xffffffffu;
+  const unsigned lane = laneid(), rd = (lane + 1) & 31;
+  payload_acc a;
+  for (unsigned todo = __ballot_sync(FULL, size); todo; todo &= todo - 1) {
+    const int j = __ffs(todo) - 1;
+    unsigned char *bp = reinterpret_cast<unsigned char *>(__shfl_sync(FULL, reinterpret_cast<unsigned long long>(p), j));
+    const uint32_t bs = __shfl_sync(FULL, size, j), bkey = __shfl_sync(FULL, key, j), bu = bs >> 4;
+    uint4 *u4 = reinterpret_cast<uint4 *>(bp);
+    for (uint32_t u = lane; u < bu; u += 32) u4[u] = pat4(bkey, 4 * u);
+    if (lane == (bu & 31) && (bs & 15)) block_rest<true>(bp, bkey, bs, a);
+    __syncwarp();
+    for (uint32_t u = rd; u < bu; u += 32) check4(__ldcg(u4 + u), pat4(bkey, 4 * u), a);
+    if (rd == (bu & 31) && (bs & 15)) block_rest<false>(bp, bkey, bs, a);
+  }
+  return a;
+}
+
+/* Mean payload units of a task's blocks up to which they are paced, on lists of
+ * pages: 24 unstaged (2^20 requests of 256 B: 193 to 1380 us from run to run,
+ * paced 216; of 384 B 230 to 990, paced 227; any size up to 600 B 290, and up to
+ * 1300 where the host waits for every round, paced 350), 8 staged (64 B: 266 to
+ * 1290, paced 222; 256 B 188, paced 227). */
+__host__ __device__ constexpr unsigned pace_payload(int v, bool stage) {
+  return v != OURO_PAGE_VLIST ? 0u : stage ? 8u : 24u;
+}
+
+/* PACE: see pace_payload (0: not); only where the warp's tasks have 16 requests
+ * or more (wide), as in every large batch. */
+template <int OP, unsigned PACE = 0>
 __device__ __forceinline__ void warp_payload(unsigned char *p, uint32_t size, uint32_t tid, uint32_t seed, int mode,
-                                             payload_acc &a) {
+                                             payload_acc &a, bool wide = false) {
   constexpr unsigned FULL = 0xffffffffu;
   const unsigned lane = laneid();
   if (mode == 0) {
@@ -295,6 +330,14 @@ __device__ __forceinline__ void warp_payload(unsigned char *p, uint32_t size, ui
   const uint32_t units = size >> 4;
   const bool flat = units <= pay_flat(OP);
   if (OP & PAY_CHECK) a.words += (size >> 2) + ((size & 3) != 0);
+  if (OP == PAY_FUSED && PACE && wide &&
+      __reduce_add_sync(FULL, units < 32u * PACE ? units : 32u * PACE) < PACE * __popc(__ballot_sync(FULL, size != 0)) + 1) {
+    const payload_acc r = payload_paced(p, size, key);
+    a.mism += r.mism;
+    a.x ^= r.x;
+    a.s += r.s;
+    return;
+  }
   if (__any_sync(FULL, (flat && units) || (size & 15))) {
     const payload_acc r = payload_row<OP>(p, size, key, flat ? units : 0);
     a.mism += r.mism;
