@@ -85,7 +85,8 @@ k_batches_persistent(ouro_heap_dev h, const uint32_t *sizes, const unsigned long
     else p = static_cast<unsigned char *>(malloc_v<V>(h, sz, active));
     if (active && !p) nulls++;
     __syncwarp();
-    warp_payload<PAY_FUSED, pace_payload(V, STAGE)>(p, sz, (uint32_t)i, seed + b, mode, a, round_log >= 4);
+    warp_payload<PAY_FUSED, plain_payload(V, STAGE), pace_payload(V, STAGE)>(p, sz, (uint32_t)i, seed + b, mode, a,
+                                                                             round_log >= 4);
     __syncwarp();
     if (STAGE) ouro::detail::stage_free<V, 8>(ctx, h, p, __activemask(), p ? size_class(h, sz) : -1);
     else free_v<V>(h, p);
@@ -120,7 +121,7 @@ ouro_status batches_form(ouro_heap *H, const uint32_t *d_sizes, const unsigned l
   const int grid = std::max(1, persistent_blocks_per_sm<V, STAGE>(blocks_per_sm)) * ouro::host::sm_count();
   const unsigned long long warps = 8ull * grid, requests = n_tasks << TASK_REQ_LOG;
   unsigned round_log = 0;
-  for (unsigned t = ouro::host::round_task(requests, warps, ouro_page_queues(V)); t > 1; t >>= 1) ++round_log;
+  for (unsigned t = ouro::host::round_task(requests, warps, ouro_page_queues(V), STAGE); t > 1; t >>= 1) ++round_log;
   /* single rounds for the last two tasks' worth per warp */
   const unsigned long long rounds = requests >> round_log, tail = (2 * warps) << (TASK_REQ_LOG - round_log);
   k_batches_persistent<V, STAGE><<<grid, 256, 0, s>>>(H->d, d_sizes, d_offs, d_task_offs, n_batches, seed, mode, d_out,

@@ -48,16 +48,22 @@ ouro_status round_fused_on(ouro_heap *H, const uint32_t *d_sizes, size_t n, uint
  * to eight requests per warp go out as one task each (32 batches of 256 to
  * 8192 requests: 62 us a round with tasks of 32, 11 so).  Beyond that a warp
  * gets at least four tasks, so that the last ones fill the gaps, of at least
- * eight requests, which share their queue atomics.  On chunk queues the steps
+ * eight requests, which share their queue atomics.  Without a stage every
+ * request goes to its queue, so there up to 16 requests share a task at once,
+ * and 32 as soon as that leaves one and a half tasks per warp (page array,
+ * tasks of 8 / 16 / 32: 110,000 sizes up to 4096 B 79 / 78 / 72 us, up to 8192
+ * B 111 / 118 / 106, 262,144 of the size sweep 135 / 126 / 113, up to 8192 B 231
+ * / 223 / 237; 200,000 up to 8192 B 185 / 180 / 210).  On chunk queues the steps
  * that a task's requests share (pop, reserve, claim, queue again) cost more
  * than uneven ends do, so their tasks go up to 32 requests first, with half
  * of the warps idle if need be (200,003 requests on the staged virtualized
  * array: tasks of 16 153 us, of 32 140; 30,011 on the chunk array: tasks of 16
  * 124 us, of 32 105; 3001: tasks of 4 56 us, of 32 80). */
-inline unsigned round_task(unsigned long long n, unsigned long long warps, bool page_queues) {
+inline unsigned round_task(unsigned long long n, unsigned long long warps, bool page_queues, bool staged) {
+  const unsigned shared = !page_queues ? 32u : staged ? 8u : 16u, rounds = !page_queues || staged ? 8 : 3;
   unsigned t = 1;
-  while (t < (page_queues ? 8u : 32u) && t * warps < (page_queues ? n : 2 * n)) t *= 2;
-  while (t < 32 && 8 * t * warps <= n) t *= 2;
+  while (t < shared && t * warps < (page_queues ? n : 2 * n)) t *= 2;
+  while (t < 32 && rounds * t * warps <= n) t *= 2;
   return t;
 }
 }  // namespace host

@@ -714,7 +714,8 @@ __global__ void __launch_bounds__(256, ouro_page_queues(V) ? OURO_FUSED_MIN_BLOC
       if (ptrs) ptrs[i] = p;
     }
     __syncwarp();
-    warp_payload<PAY_FUSED, pace_payload(V, STAGE)>(p, sz, (uint32_t)i, seed, mode, a, task >= 16);
+    warp_payload<PAY_FUSED, plain_payload(V, STAGE), pace_payload(V, STAGE)>(p, sz, (uint32_t)i, seed, mode, a,
+                                                                             task >= 16);
     __syncwarp();
     /* staged: the class of each block is known here, so the free skips the
      * chunk-table lookup (one L2 round trip per task off the warp's chain) */
@@ -882,7 +883,7 @@ template <int V, bool STAGE>
 ouro_status round_fused_form(ouro_heap *H, const uint32_t *d_sizes, size_t n, uint32_t seed, int mode,
                              ouro_check *d_out, void **d_ptrs, void *work, cudaStream_t s) {
   const int block = 256, cap = occupancy_grid(k_round_fused<V, STAGE>, block);
-  const unsigned task = ouro::host::round_task(n, (size_t)cap * (block / 32), ouro_page_queues(V));
+  const unsigned task = ouro::host::round_task(n, (size_t)cap * (block / 32), ouro_page_queues(V), STAGE);
   const int grid = grid_for((n + task - 1) / task * 32, block, cap);
   work_slot *slot = static_cast<work_slot *>(work);
   ouro::host::launch_chained(k_round_fused<V, STAGE>, grid, block, s, H->d, d_sizes, n, seed, mode, task, d_out,

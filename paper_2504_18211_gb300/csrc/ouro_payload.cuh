@@ -153,9 +153,10 @@ __device__ __forceinline__ void check4(const uint4 &got, const uint4 &want, payl
  * slots and tables).  2^20 fused size-sweep round: 326 -> 315 us; the policy
  * on the stores alone 351 us (the read-back renewed the lines), on the loads
  * alone 330.  ld.global.cg reads L2, past any line of L1. */
-__device__ __forceinline__ unsigned long long stream_policy() {
+__device__ __forceinline__ unsigned long long stream_policy(bool plain = false) {
   unsigned long long pol;
-  asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
+  if (plain) asm("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(pol));
+  else asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
   return pol;
 }
 __device__ __forceinline__ void st_stream(uint4 *p, const uint4 &v, unsigned long long pol) {
@@ -215,12 +216,13 @@ __device__ __forceinline__ unsigned row_owner(unsigned incl, unsigned f) {
 /* The row of small blocks (n_units > 0 for a lane whose block is in it) and
  * every block's rest.  Out of line: its registers (four loads in flight and
  * their places in the row) stay out of the allocating kernels' budget. */
-template <int OP>
-__device__ __noinline__ payload_acc payload_row(unsigned char *p, uint32_t size, uint32_t key, uint32_t n_units) {
+template <int OP, bool PLAIN>
+__device__ __noinline__ payload_acc payload_row(unsigned char *p, uint32_t size, uint32_t key, uint32_t n_units,
+                                                bool plain = false) {
   constexpr unsigned FULL = 0xffffffffu;
   const unsigned lane = laneid();
   const unsigned rd = OP == PAY_FUSED ? (lane + 1) & 31 : lane;   /* lane whose units this lane checks */
-  const unsigned long long pol = stream_policy();
+  const unsigned long long pol = stream_policy(PLAIN && plain);
   payload_acc a;
   uint32_t incl = n_units;
 #pragma unroll
@@ -304,9 +306,20 @@ __host__ __device__ constexpr unsigned pace_payload(int v, bool stage) {
   return v != OURO_PAGE_VLIST ? 0u : stage ? 8u : 24u;
 }
 
-/* PACE: see pace_payload (0: not); only where the warp's tasks have 16 requests
- * or more (wide), as in every large batch. */
-template <int OP, unsigned PACE = 0>
+/* Unstaged rounds on plain page arrays: pages come and go in queue order, so a
+ * page is not seen again before all others, and in a large batch neither the
+ * evict_first policy nor a row that holds less than a sixteenth of its task's
+ * units pays.  2^20 size sweep: 380 us with both, 371 without the policy, 363
+ * without either; a row of all blocks of 64 B 97 and 95 us, any size up to 600
+ * B 197 and 183.  10,240 blocks of 16 B: 14.8 us with the policy, 15.4 without.
+ * (On virtualized queues the policy is worth more than in staged rounds: 422 us
+ * with it on a list and 490 without, 340 and 424 on an array.) */
+__host__ __device__ constexpr bool plain_payload(int v, bool stage) { return v == OURO_PAGE_ARRAY && !stage; }
+constexpr uint32_t PAY_PLAIN_SHARE = 16;
+
+/* PLAIN: see plain_payload; PACE: see pace_payload (0: not).  Both only where
+ * the warp's tasks have 16 requests or more (wide), as in every large batch. */
+template <int OP, bool PLAIN = false, unsigned PACE = 0>
 __device__ __forceinline__ void warp_payload(unsigned char *p, uint32_t size, uint32_t tid, uint32_t seed, int mode,
                                              payload_acc &a, bool wide = false) {
   constexpr unsigned FULL = 0xffffffffu;
@@ -328,7 +341,11 @@ __device__ __forceinline__ void warp_payload(unsigned char *p, uint32_t size, ui
   if (!p) size = 0;
   const unsigned rd = OP == PAY_FUSED ? (lane + 1) & 31 : lane;   /* lane whose units this lane checks */
   const uint32_t units = size >> 4;
-  const bool flat = units <= pay_flat(OP);
+  bool flat = units <= pay_flat(OP);
+  if (PLAIN && OP == PAY_FUSED && wide) {
+    const uint32_t row = __reduce_add_sync(FULL, flat ? units : 0u), rest = __reduce_add_sync(FULL, flat ? 0u : units);
+    if (rest > PAY_PLAIN_SHARE * row) flat = units == 0;
+  }
   if (OP & PAY_CHECK) a.words += (size >> 2) + ((size & 3) != 0);
   if (OP == PAY_FUSED && PACE && wide &&
       __reduce_add_sync(FULL, units < 32u * PACE ? units : 32u * PACE) < PACE * __popc(__ballot_sync(FULL, size != 0)) + 1) {
@@ -339,14 +356,14 @@ __device__ __forceinline__ void warp_payload(unsigned char *p, uint32_t size, ui
     return;
   }
   if (__any_sync(FULL, (flat && units) || (size & 15))) {
-    const payload_acc r = payload_row<OP>(p, size, key, flat ? units : 0);
+    const payload_acc r = payload_row<OP, PLAIN>(p, size, key, flat ? units : 0, wide);
     a.mism += r.mism;
     a.x ^= r.x;
     a.s += r.s;
   }
 
   /* the larger blocks, one at a time */
-  const unsigned long long pol = stream_policy();
+  const unsigned long long pol = stream_policy(PLAIN && wide);
   for (unsigned big = __ballot_sync(FULL, !flat); big; big &= big - 1) {
     const int j = __ffs(big) - 1;
     uint4 *u4 = reinterpret_cast<uint4 *>(__shfl_sync(FULL, reinterpret_cast<unsigned long long>(p), j));
