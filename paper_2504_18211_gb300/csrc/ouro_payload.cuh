@@ -363,8 +363,10 @@ __device__ __forceinline__ void warp_payload(unsigned char *p, uint32_t size, ui
   }
 
   /* the larger blocks, one at a time */
+  unsigned big = __ballot_sync(FULL, !flat);
+  if (!big) return;
   const unsigned long long pol = stream_policy(PLAIN && wide);
-  for (unsigned big = __ballot_sync(FULL, !flat); big; big &= big - 1) {
+  for (; big; big &= big - 1) {
     const int j = __ffs(big) - 1;
     uint4 *u4 = reinterpret_cast<uint4 *>(__shfl_sync(FULL, reinterpret_cast<unsigned long long>(p), j));
     const uint32_t bu = __shfl_sync(FULL, units, j), bkey = __shfl_sync(FULL, key, j);
