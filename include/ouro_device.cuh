@@ -437,10 +437,10 @@ __device__ inline void seg_init(const ouro_heap_dev &h, unsigned x, unsigned idx
 }
 
 /* A fresh segment with index idx: spare of the class first, else a chunk of
- * the heap. */
-__device__ inline unsigned seg_new(const ouro_heap_dev &h, int c, unsigned idx) {
+ * the heap (fresh). */
+__device__ inline unsigned seg_new(const ouro_heap_dev &h, int c, unsigned idx, bool &fresh) {
   unsigned x = spare_pop(h, c);
-  const bool fresh = x == OURO_NIL;
+  fresh = x == OURO_NIL;
   if (fresh) {
     chunk_range r = take_chunks(h, 1);
     if (r.k1 + r.k2 == 0) return OURO_NIL;
@@ -451,6 +451,11 @@ __device__ inline unsigned seg_new(const ouro_heap_dev &h, int c, unsigned idx) 
   seg_init(h, x, idx, fresh);
   OURO_TRACE_EVENT(OURO_TR_SEGMENT, c, idx, x);
   return x;
+}
+
+__device__ inline unsigned seg_new(const ouro_heap_dev &h, int c, unsigned idx) {
+  bool fresh;
+  return seg_new(h, c, idx, fresh);
 }
 
 /* Retired list segments xs[0..k), in list order, are appended behind the
@@ -1078,10 +1083,11 @@ __device__ __forceinline__ unsigned long long *vl_slot(const ouro_heap_dev &h, i
 static __device__ __noinline__ unsigned vl_create_run(const ouro_heap_dev &h, int c, unsigned long long cur) {
   ouro_qhdr *q = qh(h, c);
   const unsigned idx = hi32(cur) + 1;
-  const unsigned long long lim = (ld_rlx(&q->tail.v) + OURO_AHEAD_POS) / h.seg_cap;
   unsigned xs[OURO_VL_RUN], k = 1;
-  xs[0] = seg_new(h, c, idx);
+  bool fresh;
+  xs[0] = seg_new(h, c, idx, fresh);
   if (xs[0] == OURO_NIL) return OURO_NIL;
+  const unsigned long long lim = fresh ? 0 : (ld_rlx(&q->tail.v) + OURO_AHEAD_POS) / h.seg_cap;   /* fresh: no spares */
   for (; k < OURO_VL_RUN && idx + k <= lim; ++k) {
     const unsigned x = spare_pop(h, c);
     if (x == OURO_NIL) break;
