@@ -7,13 +7,24 @@
 #include "ouro.h"
 #include "ouro_device.cuh"
 
-/* Ring slack: at most this many threads can be resident on the GPU at once
- * (152 SMs x 2048), so a ring of (capacity + slack) slots never makes a
- * producer wait for a consumer that is still in flight one lap behind. */
-#define OURO_RING_SLACK (1ull << 19)
-/* virtualized-array directories also span positions that are waiting for a
- * producer or in flight (more than twice the resident threads of 152 SMs) */
-#define OURO_VA_SLACK (1ull << 20)
+/* Queue positions that kernels can hold at once on the GPU's 152 SMs: one per
+ * resident thread (2048 an SM) in most kernels, four per thread in those of
+ * large batches.  The batch malloc has 64 registers a thread, 1024 threads an SM
+ * (its launch bounds; fewer registers would leave more threads resident). */
+#define OURO_SMS 152ull
+#define OURO_BATCH_POS 4ull
+#define OURO_BATCH_MALLOC_THREADS 1024ull
+/* Ring slack: at least the positions that consumers can hold, so that a ring of
+ * (capacity + slack) slots does not make a producer wait for a consumer that is
+ * still in flight one lap behind.  (Such a wait is bounded and ends when the
+ * consumer gets on, so this is about time.) */
+#define OURO_RING_SLACK (5ull << 17)
+static_assert(OURO_RING_SLACK >= OURO_SMS * 2048 && OURO_RING_SLACK >= OURO_SMS * OURO_BATCH_MALLOC_THREADS * OURO_BATCH_POS,
+              "ring slack below the positions in flight");
+/* Virtualized-array directories also span positions that are waiting for a
+ * producer or in flight: four per thread, whatever kernel holds them. */
+#define OURO_VA_SLACK (19ull << 16)
+static_assert(OURO_VA_SLACK >= OURO_SMS * 2048 * OURO_BATCH_POS, "directory slack below the positions in flight");
 /* work slots of fused rounds: one per stream that launches them on a heap (up
  * to this many), each on its own 128-byte line; zero between launches */
 #define OURO_WORK_SLOTS 64

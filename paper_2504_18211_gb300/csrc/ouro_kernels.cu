@@ -162,7 +162,7 @@ __device__ __noinline__ void blk_free_rest(const ouro_heap_dev &h, int cls, unsi
 }
 
 template <int V, int R>
-__global__ void __launch_bounds__(256, 4) k_batch_malloc_blk(ouro_heap_dev h, const uint32_t *sizes, void **ptrs,
+__global__ void __launch_bounds__(256, OURO_BATCH_MALLOC_THREADS / 256) k_batch_malloc_blk(ouro_heap_dev h, const uint32_t *sizes, void **ptrs,
                                                              size_t n) {
   ouro::chain_begin();
   constexpr int QF = ouro_qform(V);
@@ -796,6 +796,7 @@ namespace launch {
  * tried together) once a batch fills every SM with four per thread; one
  * otherwise, so that a small batch still spreads over many blocks. */
 constexpr int BLK_WIDE = 4;
+static_assert(BLK_WIDE <= (int)OURO_BATCH_POS, "the queues' slack counts on it");
 inline bool blk_wide(size_t n) { return n >= (size_t)BLK_WIDE * 256 * ouro::host::sm_count(); }
 /* The plain-array batch free takes eight requests per thread in blocks of
  * 128 once a batch fills every SM with four such blocks: a 2^20 batch then
