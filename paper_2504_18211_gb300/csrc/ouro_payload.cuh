@@ -72,17 +72,12 @@ __device__ __forceinline__ void free_v(const ouro_heap_dev &h, void *p, int know
   }
 }
 
-/* Staged malloc / free: the warp's shared-memory stacks first (every queue
- * form), then the heap. */
+/* Staged malloc: the warp's shared-memory stacks first (every queue form), then
+ * the heap. */
 template <int V, int WARPS>
 __device__ __forceinline__ void *stage_malloc_v(ouro_block_ctx<WARPS> &ctx, const ouro_heap_dev &h,
                                                 unsigned long long n, bool want) {
   return ouro::detail::stage_malloc<V, WARPS>(ctx, h, n, want);
-}
-
-template <int V, int WARPS>
-__device__ __forceinline__ void stage_free_v(ouro_block_ctx<WARPS> &ctx, const ouro_heap_dev &h, void *p) {
-  ouro::detail::stage_free<V, WARPS>(ctx, h, p);
 }
 
 /* ------------------------------------------------------------- payload */
