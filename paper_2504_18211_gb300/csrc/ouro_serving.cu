@@ -53,7 +53,8 @@ struct serve_args {
   unsigned long long *tables;    /* n_slots x max_blocks block pointers */
   /* results */
   unsigned long long *sess_out;  /* per session: xor, sum, mismatches, admit step, done step (u64 each) */
-  unsigned long long *step_ns;   /* per step: %globaltimer after admission, growth and completion (3 words) */
+  unsigned long long *step_ns;   /* per step: %globaltimer when its growth begins, when that has ended, and
+                                    when its frees and the next admission have (3 words) */
   unsigned long long *ctl;       /* [0] barrier arrivals, [1] reserved, [2] next arrival,
                                     [3] committed blocks, [4] error, [5] mallocs, [6] frees, [7] failed,
                                     [8] free-slot stack top, [9 + step % 2] sessions finished this step */
@@ -135,6 +136,36 @@ __device__ void serve_admit(const serve_args &A, uint32_t step) {
  * 17 at the copy rate). */
 constexpr uint32_t SERVE_PIECE = 256;
 
+/* One block of class cls for every lane with `want` (all 32 lanes call).  On
+ * chunk queues the warp pops a chunk per lane at once, as the batch malloc
+ * does: one class group of chunk_malloc pops them one after another, and a
+ * serving block takes a chunk of its own where chunks are no larger (400 steps
+ * of about 1700 blocks: chunk array 15.7 ms, 9.3 so, virtualized list 20.2 and
+ * 12.3). */
+template <int V>
+__device__ __forceinline__ unsigned char *serve_malloc(const ouro_heap_dev &h, uint32_t bytes, bool want) {
+  if constexpr (!ouro_page_queues(V)) {
+    if (!h.deopt) {
+      __shared__ unsigned items[32];
+      const unsigned wm = __ballot_sync(0xffffffffu, want), need = __popc(wm), rank = __popc(wm & lanemask_lt());
+      if (!need) return nullptr;
+      const int cls = size_class(h, bytes);
+      const unsigned got = chunk_acquire<V>(h, cls, need, items);
+      __syncwarp();
+      const unsigned item = want && rank < got ? items[rank] : OURO_NIL;
+      const unsigned n = __popc(__ballot_sync(0xffffffffu, item != OURO_NIL));
+      if (laneid() == 0) {
+        stat_add(h, cls, OURO_ST_MALLOC, n);
+        stat_add(h, cls, OURO_ST_FAILED, need - n);
+      }
+      return item != OURO_NIL ? h.base + ((size_t)item << (4 + cls)) : nullptr;
+    }
+  }
+  /* (a step's growth can carve thousands of chunks: eight slot writes per
+   *  lane in flight while the warp fills them) */
+  return static_cast<unsigned char *>(malloc_v<V, 8>(h, bytes, want));
+}
+
 /* a lane's session between two steps of one launch */
 struct serve_lane {
   unsigned long long x, sum, mism;
@@ -188,10 +219,8 @@ __device__ void serve_grow(const serve_args &A, uint32_t step, serve_lane *keep)
         }
       }
       __syncwarp();
-      /* (a step's growth can carve thousands of chunks: eight slot writes per
-       *  lane in flight while the warp fills them) */
       const bool want = sess >= 0 && k < total;
-      unsigned char *bp = static_cast<unsigned char *>(malloc_v<V, 8>(h, A.block_bytes, want));
+      unsigned char *bp = serve_malloc<V>(h, A.block_bytes, want);
       __syncwarp();
       grown = want && bp;
       const unsigned gm = __ballot_sync(0xffffffffu, grown), wm = __ballot_sync(0xffffffffu, want);
