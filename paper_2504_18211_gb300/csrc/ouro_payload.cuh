@@ -414,21 +414,22 @@ __device__ inline void block_acc(payload_acc &a, unsigned long long nulls, unsig
   __syncthreads();
 }
 
-/* A block's counters (block_acc) added to *out, which was zero when the
- * kernel began.  The words are 32-bit, so their XOR only ever touches the low
- * half of xor64; the high half may hold a fused round's task counter. */
-__device__ __forceinline__ void add_check(const unsigned long long (&sm)[5], ouro_check *out) {
-  if (sm[0]) atomicAdd(&out->nulls, sm[0]);
-  if (sm[1]) atomicAdd(&out->mismatches, sm[1]);
-  atomicXor(reinterpret_cast<unsigned *>(&out->xor64), (unsigned)sm[2]);
-  atomicAdd(&out->sum64, sm[3]);
-  atomicAdd(&out->words, sm[4]);
+/* A block's counters (block_acc) added to acc, the five words of an ouro_check
+ * in their order.  The words checked are 32-bit, so their XOR only ever touches
+ * the low half of its word; the high half may hold a fused round's task
+ * counter. */
+__device__ __forceinline__ void add_check(const unsigned long long (&sm)[5], unsigned long long *acc) {
+  if (sm[0]) atomicAdd(&acc[0], sm[0]);
+  if (sm[1]) atomicAdd(&acc[1], sm[1]);
+  atomicXor(reinterpret_cast<unsigned *>(&acc[2]), (unsigned)sm[2]);
+  atomicAdd(&acc[3], sm[3]);
+  atomicAdd(&acc[4], sm[4]);
 }
 
 __device__ inline void flush_acc(payload_acc &a, unsigned long long nulls, ouro_check *out) {
   __shared__ unsigned long long sm[5];
   block_acc(a, nulls, sm);
-  if (threadIdx.x == 0) add_check(sm, out);
+  if (threadIdx.x == 0) add_check(sm, reinterpret_cast<unsigned long long *>(out));
 }
 
 /* A work slot (a 128-byte line): all zero between launches, and never used by
@@ -445,13 +446,9 @@ struct work_slot {
 __device__ inline void finish_acc(payload_acc &a, unsigned long long nulls, work_slot *w, ouro_check *out) {
   __shared__ unsigned long long sm[5];
   block_acc(a, nulls, sm);
-  if (threadIdx.x == 0 && !w) add_check(sm, out);
-  if (threadIdx.x == 0 && w) {
-    if (sm[0]) atomicAdd(&w->acc[0], sm[0]);
-    if (sm[1]) atomicAdd(&w->acc[1], sm[1]);
-    atomicXor(&w->acc[2], sm[2]);
-    atomicAdd(&w->acc[3], sm[3]);
-    atomicAdd(&w->acc[4], sm[4]);
+  if (threadIdx.x == 0) {
+    add_check(sm, w ? w->acc : reinterpret_cast<unsigned long long *>(out));
+    if (!w) return;
     __threadfence();
     if (atomicAdd(&w->done, 1ull) == gridDim.x - 1) {
       __threadfence();
