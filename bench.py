@@ -79,8 +79,8 @@ def dist_env():
 # from the sources whose digest is recorded; null once they change.
 FUSED_KERNEL_SOURCES = ("include/ouro_device.cuh", "paper_2504_18211_gb300/csrc/ouro_payload.cuh",
                         "paper_2504_18211_gb300/csrc/ouro_kernels.cu", "paper_2504_18211_gb300/csrc/ouro_internal.cuh")
-FUSED_TRAFFIC = {"sources_sha256": "8fd89ca53171beef4b24fce5813c76db6a7e924fe5ec6114411f268fae08ce19",
-                 "bytes_per_launch": 1712762624}
+FUSED_TRAFFIC = {"sources_sha256": "fe1e6752879b808f6c972d951d95e9737fbf399e182df7fb0df8d74494587fa5",
+                 "bytes_per_launch": 1713373440}
 
 
 def kernel_sources_digest() -> str:

@@ -52,7 +52,7 @@ enum {
  *                       position order, found by a walk (with a lookaside);
  *   virtualized array:  slots live in heap chunks found by index through a
  *                       per-class directory of 8-B entries, next_pow2 of
- *                       ceil((bytes/page + 2^20) / segment slots) + 4
+ *                       ceil((bytes/page + 19 * 2^16) / segment slots) + 4
  *                       entries (chunk queues: n_chunks in place of
  *                       bytes/page).  A segment returns to its class's spare
  *                       stack once all its positions are produced and
@@ -273,7 +273,8 @@ ouro_status ouro_heap_stats_static(ouro_heap *h, ouro_stats *out, void *stream);
 /* One kernel for n_batches batches (Sec. 3 driver round per request):
  * request i of batch b (d_sizes[d_offs[b] + i]) allocates, writes its
  * pattern (seed + b, thread id i), reads it back and frees.  Warps pull
- * 256-request tasks from *d_work (device scratch, 1 word, reset here);
+ * tasks of 256 requests, and shorter rounds at the end of the pass, from
+ * *d_work (device scratch, 1 word, reset here);
  * d_task_offs[b] = sum over batches before b of ceil(count/256), n_tasks
  * its total.  d_out: n_batches checks (overwritten).  blocks_per_sm <= 0:
  * the occupancy limit.  d_offs, d_task_offs: device arrays of n_batches+1. */
@@ -290,7 +291,8 @@ int ouro_batches_max_blocks_per_sm(const ouro_heap *h);
  * form 0: ouro_round_fused per batch; form 1: ouro_batch_malloc,
  * ouro_pattern_write, ouro_pattern_check, ouro_batch_free per batch (d_ptrs:
  * device scratch for the largest batch).  h_offs: HOST offsets (n_batches+1).
- * Replay with ouro_batch_graph_launch; the captured pointers must stay valid. */
+ * Replay with ouro_batch_graph_launch; the captured pointers must stay valid.
+ * ouro_batch_graph_destroy waits for the replays in flight. */
 typedef struct ouro_batch_graph ouro_batch_graph;
 ouro_status ouro_batch_graph_create(ouro_heap *h, const uint32_t *d_sizes, const unsigned long long *h_offs,
                                     uint32_t n_batches, uint32_t seed, int mode, ouro_check *d_out,

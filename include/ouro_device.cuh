@@ -1197,7 +1197,7 @@ static __device__ __noinline__ unsigned long long *vl_slot_walk(const ouro_heap_
  * from the heap at once, set up by all lanes and linked behind the back as one
  * chain, instead of by one lane in turn, a walk, a chunk and a thousand cells
  * each.  With it and the tail rule of page_malloc the first burst on a cold
- * list (3 * 2^18 requests, 25.4 ms) takes no longer in the block kernels'
+ * list (3 * 2^18 requests, 25.6 ms) takes no longer in the block kernels'
  * four-request form than it did with one request per thread; without the two
  * 27.9.  Leaves the rest (a single segment, the first one, spares) to
  * vl_slot. */

@@ -5,7 +5,8 @@ writes its pattern, reads it back and frees):
   per_launch4  four library launches per batch (malloc, write, check, free)
   per_launch1  one fused-round launch per batch
   graph        the per-batch fused launches captured once as a CUDA graph
-  persistent   one kernel for all batches, 256-request tasks from a device counter
+  persistent   one kernel for all batches, tasks of 256 requests and at the end
+               of a pass single rounds of 32 or fewer from a device counter
 Only marshalling and timing happen here; every step runs in libouro.so.
 """
 from __future__ import annotations

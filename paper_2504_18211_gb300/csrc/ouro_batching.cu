@@ -7,9 +7,11 @@
  *   - per launch:  one fused-round launch per batch (ouro_round_fused), or
  *                  four launches per batch (malloc / write / check / free);
  *   - CUDA graph:  the per-batch launches captured once and replayed;
- *   - persistent:  ONE kernel for all batches; warps pull 256-request tasks
- *                  from a device work counter, so uneven batches overlap
- *                  and the allocator state never leaves L2 between them.
+ *   - persistent:  ONE kernel for all batches; warps pull tasks of 256
+ *                  requests, and single rounds of 32 or fewer at the end of
+ *                  a pass, from a device work counter, so uneven batches
+ *                  overlap and the allocator state never leaves L2 between
+ *                  them.
  * Request i of batch b uses pattern seed (seed + b) and thread id i (its
  * index inside the batch), in every form, so the per-batch checks agree.
  */
@@ -32,7 +34,8 @@ constexpr unsigned TASK_REQ_LOG = 8;   /* 256 requests per persistent task (the 
  * task may have empty rounds).  A claim is a whole task until `last_wave`,
  * then one round: with whole tasks to the end a warp had 4 or 5 of them on a
  * pass of 6 M requests, and the kernel ended with the fives (96 batches of up
- * to 2^18 requests, staged: 3.22 ms, 3.05 so). */
+ * to 2^18 requests, staged: 3.22 ms, 3.05 so on one box; whole passes differ by
+ * a tenth from box to box, 3.05 to 3.44 ms since). */
 template <int V, bool STAGE>
 __global__ void __launch_bounds__(256, ouro_page_queues(V) ? 4 : 2)   /* chunk queues: no spills at 2 per SM */
 k_batches_persistent(ouro_heap_dev h, const uint32_t *sizes, const unsigned long long *offs,

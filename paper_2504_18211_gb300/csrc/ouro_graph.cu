@@ -81,8 +81,9 @@ constexpr unsigned LANE_COPY = 32;      /* entries of a list that its grower's l
  * reservation, the writes and their commit, about three dependent L2 round
  * trips; what is left to wait for is looked at once a round.  A warp per run
  * under the vertex's lock took about 5 us for each run and one atomic on the
- * appended count per run: 2^22 edges on 2^18 vertices 5570 us, 660 so (what
- * bounds it now is the chain of the largest list's segments).  Adds the lane's
+ * appended count per run: 2^22 edges on 2^18 vertices 5570 us, 660 so (with
+ * uniform sources 580: what bounds it is the chain of each warp's 32 runs,
+ * about 16 us, and not the largest list).  Adds the lane's
  * entries written, dropped (no memory) and skipped (a wait ran out). */
 template <int V>
 __device__ void warp_append(const ouro_heap_dev &h, vertex *vx, const unsigned *from, unsigned n, unsigned &written,

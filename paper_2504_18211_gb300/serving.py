@@ -62,8 +62,8 @@ class ServeRun:
         ns = self.step_ns.cpu().numpy().view(np.uint64).astype(np.int64).reshape(-1, 3)
         ends = ns[:, 2]
         lat = np.diff(ends) / 1e3 if ends.size > 1 else np.zeros(0)
-        phases = {"admit_us": (ns[1:, 0] - ends[:-1]) / 1e3, "grow_us": (ns[1:, 1] - ns[1:, 0]) / 1e3,
-                  "complete_us": (ns[1:, 2] - ns[1:, 1]) / 1e3}
+        # growth, in which sessions also complete; then their frees, beside the next step's admission
+        phases = {"grow_us": (ns[1:, 1] - ns[1:, 0]) / 1e3, "free_admit_us": (ns[1:, 2] - ns[1:, 1]) / 1e3}
         never = np.uint64(0xFFFFFFFFFFFFFFFF)
         return {"xor": so[:, 0], "sum": so[:, 1], "mism": so[:, 2],
                 "admit": np.where(so[:, 3] == never, -1, so[:, 3].astype(np.int64)),
