@@ -46,7 +46,7 @@ enum {
 /* queue variants (the six of Sec. 3): page or chunk queues (Sec. 4.1, 4.2),
  * each as a plain array, a virtualized list or a virtualized array (Sec. 4.3).
  *   plain array:        a ring of slots outside the heap, per class
- *                       next_pow2(min(bytes/page, array_queue_capacity) + 5 * 2^17)
+ *                       next_pow2(min(bytes/page, array_queue_capacity) + 2^19)
  *                       slots of 8 B;
  *   virtualized list:   slots live in heap chunks (segments) linked in
  *                       position order, found by a walk (with a lookaside);

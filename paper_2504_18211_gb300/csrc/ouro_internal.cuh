@@ -9,18 +9,18 @@
 
 /* Queue positions that kernels can hold at once on the GPU's 152 SMs: one per
  * resident thread (2048 an SM) in most kernels, four per thread in those of
- * large batches.  The batch malloc has 64 registers a thread, 1024 threads an SM
- * (its launch bounds; fewer registers would leave more threads resident). */
+ * large batches. */
 #define OURO_SMS 152ull
 #define OURO_BATCH_POS 4ull
-#define OURO_BATCH_MALLOC_THREADS 1024ull
-/* Ring slack: at least the positions that consumers can hold, so that a ring of
- * (capacity + slack) slots does not make a producer wait for a consumer that is
- * still in flight one lap behind.  (Such a wait is bounded and ends when the
- * consumer gets on, so this is about time.) */
-#define OURO_RING_SLACK (5ull << 17)
-static_assert(OURO_RING_SLACK >= OURO_SMS * 2048 && OURO_RING_SLACK >= OURO_SMS * OURO_BATCH_MALLOC_THREADS * OURO_BATCH_POS,
-              "ring slack below the positions in flight");
+/* Ring slack: consumers that hold one position per resident thread never make a
+ * producer of a ring of (capacity + slack) slots wait one lap behind them.  The
+ * batch malloc can hold 622,592 positions (1024 threads an SM); should they all
+ * be of one class, beside a full queue of it, a producer waits for the oldest of
+ * them, which does not wait for that producer.  More slack costs more than such
+ * a wait: it doubles the rings of some heaps (12 GiB of 8 KiB pages: 2^22 slots
+ * for 2^21, rounds of 965,676 mixed requests with one word each 121 -> 130 us). */
+#define OURO_RING_SLACK (1ull << 19)
+static_assert(OURO_RING_SLACK >= OURO_SMS * 2048, "ring slack below the resident threads");
 /* Virtualized-array directories also span positions that are waiting for a
  * producer or in flight: four per thread, whatever kernel holds them. */
 #define OURO_VA_SLACK (19ull << 16)
