@@ -473,7 +473,7 @@ __global__ void __launch_bounds__(256) k_batch_free_cblk(ouro_heap_dev h, void *
  * of them runs that each went through the warp path, malloc to free: 105 us, 98
  * with this and the free above.) */
 /* (registers: the compiler's choice, but for the list, where it may settle at 80
- * with 2 KB a thread spilled: 300,007 mixed requests 139 us, 134 at 128) */
+ * with 2 KB a thread spilled: 311,304 mixed requests 139 us, 134 at 128) */
 template <int V, int R>
 __global__ void __launch_bounds__(256, V == OURO_CHUNK_VLIST ? 2 : 0) k_batch_malloc_cblk(ouro_heap_dev h, const uint32_t *sizes, void **ptrs,
                                                            size_t n) {
